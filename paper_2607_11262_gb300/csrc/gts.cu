@@ -9,6 +9,10 @@
 // graph is shared read-only by all points.  Per point, a global scratch row
 // holds the dependency counters of nodes that are not warp heads yet.
 //
+// Two kernels do this: k_simulate issues one node per step of the warp, and
+// k_simulate_lanes one node on each of up to 32 simulated SMs, where the graph and
+// the rows allow it (described above its functions; the notes here are k_simulate's).
+//
 // Semantics are those stated in include/gts.h.  Design notes:
 //  * Issue keys (Section 5.3, lowest-id reading).  A head's key is the
 //    earliest cycle >= now at which its predecessors are released and its
@@ -121,6 +125,11 @@ gts_status cuda_fail(cudaError_t e, const char *what) {
   return fail(GTS_ERR_CUDA, (const char *)buf);
 }
 
+// sums of work kept for the cost of a row: bytes to and from memory, shared-memory bytes, FMAs, elementwise ops
+enum : uint32_t { WK_MEM = 0, WK_SMEM, WK_FMA, WK_EW, WK_N };
+// per node type, its sum (7: none)
+constexpr uint32_t TYPE_WORK = 0x17703210u;
+
 // ----------------------------------------------------------------- device graph
 struct DevGraph {
   const uint4 *rec;            // [n] x=work y=lat_extra z=next node of the stream w=type | indegree<<4
@@ -133,6 +142,8 @@ struct DevGraph {
   const uint32_t *cta_off;     // [G+1]
   uint32_t W, G, row_nodes, row_ctas, cross_cta;
   uint32_t n_tiles;     // tile ids of LOAD/STORE nodes (rng.x = tile + 1; 0: none)
+  float work[WK_N];     // work summed over the stack, per rate
+  uint32_t zero_types;  // bit k: some node of type k has no work (or is a NOP) and no extra latency
   uint32_t class_mask;  // bit r < 5: some node uses per-SM class r; CM_NOC: some node crosses the NoC
 };
 
@@ -970,6 +981,35 @@ __device__ __forceinline__ uint32_t first_point_of(const uint32_t *order, uint32
   return next_point_of(order, n_order, counter, first, n, 0u, 0u, lane);
 }
 
+// A row's derived constants: division constants of its rates, base latencies per
+// type and the two LOAD bases of the L2 model.  All lanes call it.
+__device__ __forceinline__ void put_constants(uint32_t *sp, const int32_t *prm, int lane) {
+  if (lane < (int)RC_N) {
+    *reinterpret_cast<uint64_t *>(sp + O_MAG + 2 * lane) = div_const((uint32_t)prm[GTS_P_HBM_BPC + 2 * lane]);
+  } else if (lane == (int)RC_N) {
+    *reinterpret_cast<uint64_t *>(sp + O_MAG + 10) = div_const((uint32_t)prm[GTS_P_NOC_BPC]);
+  } else if (lane == (int)RC_N + 1) {
+    *reinterpret_cast<uint64_t *>(sp + O_MAG + 12) = div_const((uint32_t)prm[GTS_P_L2_BPC]);
+  } else if (lane == 30) {  // LOAD base with the L2 model: hit, miss
+    sp[O_L2B] = (uint32_t)prm[GTS_P_TMA_LAT] + (uint32_t)prm[GTS_P_L2_LAT];
+    sp[O_L2B + 1] = (uint32_t)prm[GTS_P_TMA_LAT] + (uint32_t)prm[GTS_P_L2_LAT] + (uint32_t)prm[GTS_P_DRAM_LAT];
+  }
+  if (lane < 8) {  // base latency per type: LOAD, SMEM, MMA, EW, STORE, BAR, NOP
+    uint32_t bl = 0;
+    switch (lane) {
+      case GTS_LOAD: bl = (uint32_t)prm[GTS_P_TMA_LAT] + (uint32_t)prm[GTS_P_DRAM_LAT]; break;
+      case GTS_SMEM: bl = (uint32_t)prm[GTS_P_SMEM_LAT]; break;
+      case GTS_MMA: bl = (uint32_t)prm[GTS_P_MMA_LAT]; break;
+      case GTS_EW: bl = (uint32_t)prm[GTS_P_ALU_LAT]; break;
+      case GTS_STORE: bl = (uint32_t)prm[GTS_P_TMA_LAT]; break;
+      case GTS_BAR: bl = (uint32_t)prm[GTS_P_BAR_LAT]; break;
+      case GTS_DSMEM: bl = (uint32_t)prm[GTS_P_SMEM_LAT] + (uint32_t)prm[GTS_P_NOC_LAT]; break;
+      default: break;
+    }
+    sp[O_BASE + lane] = bl;
+  }
+}
+
 // EXT: the kernel instance that also runs the per-subpartition issue policies
 // and the NoC of DSMEM nodes; the host launches a plain instance when no row
 // asks for a policy and the graph has no DSMEM node.  SPL: the plain instance
@@ -1061,30 +1101,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
         off += c;
       }
     }
-    if (lane < (int)RC_N) {
-      *reinterpret_cast<uint64_t *>(sp + O_MAG + 2 * lane) = div_const((uint32_t)prm[GTS_P_HBM_BPC + 2 * lane]);
-    } else if (lane == (int)RC_N) {
-      *reinterpret_cast<uint64_t *>(sp + O_MAG + 10) = div_const((uint32_t)prm[GTS_P_NOC_BPC]);
-    } else if (lane == (int)RC_N + 1) {
-      *reinterpret_cast<uint64_t *>(sp + O_MAG + 12) = div_const((uint32_t)prm[GTS_P_L2_BPC]);
-    } else if (lane == 30) {  // LOAD base with the L2 model: hit, miss
-      sp[O_L2B] = (uint32_t)prm[GTS_P_TMA_LAT] + (uint32_t)prm[GTS_P_L2_LAT];
-      sp[O_L2B + 1] = (uint32_t)prm[GTS_P_TMA_LAT] + (uint32_t)prm[GTS_P_L2_LAT] + (uint32_t)prm[GTS_P_DRAM_LAT];
-    }
-    if (lane < 8) {  // base latency per type: LOAD, SMEM, MMA, EW, STORE, BAR, NOP
-      uint32_t bl = 0;
-      switch (lane) {
-        case GTS_LOAD: bl = (uint32_t)prm[GTS_P_TMA_LAT] + (uint32_t)prm[GTS_P_DRAM_LAT]; break;
-        case GTS_SMEM: bl = (uint32_t)prm[GTS_P_SMEM_LAT]; break;
-        case GTS_MMA: bl = (uint32_t)prm[GTS_P_MMA_LAT]; break;
-        case GTS_EW: bl = (uint32_t)prm[GTS_P_ALU_LAT]; break;
-        case GTS_STORE: bl = (uint32_t)prm[GTS_P_TMA_LAT]; break;
-        case GTS_BAR: bl = (uint32_t)prm[GTS_P_BAR_LAT]; break;
-        case GTS_DSMEM: bl = (uint32_t)prm[GTS_P_SMEM_LAT] + (uint32_t)prm[GTS_P_NOC_LAT]; break;
-        default: break;
-      }
-      sp[O_BASE + lane] = bl;
-    }
+    put_constants(sp, prm, lane);
     for (uint32_t i = lane; i < P.L.S; i += 32) {
       uint32_t *sl = P.slot(i);
       sl[F_HID] = NONE;
@@ -1441,6 +1458,884 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
   }
 }
 
+// ----------------------------------------------------------------- lane-parallel instance
+// k_simulate_lanes: one warp per design point, one simulated SM per lane at a time.
+//
+// Without edges between CTAs an SM's schedule depends on the others only through
+// the HBM servers and the CTA slots.  With node ids in CTA order (CTAs launch in
+// id order, so a new CTA's ids exceed every resident one's) and no zero-latency
+// node, the serial schedule issues in ascending (cycle, id), and a launch at cycle
+// T comes from retirements of nodes issued before T.  So the warp keeps only two
+// things in global order and lets every SM run ahead on its own:
+//  * HBM grants.  A waiting LOAD or STORE (an SM's first by (max(key, H), id), H
+//    the earliest free HBM server) gets its server when it precedes, in (cycle,
+//    id) order, every other SM's bound on HBM heads it has not shown yet: an SM
+//    with an issuable other head at k cannot show one before max(k, its TMA's
+//    first free cycle, H), nor one with an id below its oldest CTA's; one with a
+//    finished CTA not before that CTA's retirement.  An SM whose next event is its
+//    own waiting HBM head shows nothing before that head is granted.
+//  * CTA launches.  The earliest retirement T launches once no SM's next event
+//    comes before T (a node issued at T or later retires after T).
+// Every other head issues as soon as it precedes its SM's own waiting HBM head
+// and does not pass the retirement of a CTA on its SM.  Each step of the warp
+// looks over the SMs' records, grants all it can, then issues one node on each of
+// up to 32 SMs, one per lane, and repeats that on the SMs that can go on while
+// half of them can.
+//
+// What bounds it: a step is some 1,000 dependent instructions of one warp at about
+// 4.4 cycles each (fixed-latency waits; 32% of the issue slots at 7 warps per SM),
+// for 5 to 25 nodes where k_simulate spends 500 for one.  Measured, one GB300 at
+// 2,070 MHz, ms per batch, k_simulate then this: ws GEMM 4096x4096x2048 on 3,000
+// rows 324 and 64; FlashAttention of 54,528 nodes on 257 rows 86.5 and 17.1; decoder
+// layer of 84,672 nodes on 300 rows 128 and 32.7; GEMM 512^3 on one row 3.03 and
+// 0.55, on 64 rows 3.43 and 1.00.  73.6 warp-instructions per node on the profiling
+// case (497 before).
+constexpr uint32_t LANE_SLOT_WORDS = 8;   // rdy, meta, tag, next of stream; occ, HBM occ (else servers of its class), succ
+                                          // begin, latency
+constexpr uint32_t LANE_SM_WORDS = 8;     // see lane_refresh
+constexpr uint32_t LANE_CHUNKS = 5;       // SMs a lane looks after
+constexpr uint32_t LANE_MAX_SMS = 32 * LANE_CHUNKS;
+constexpr uint32_t LANE_MAX_SLOTS = 32;   // warp slots per SM: five bits of a tag
+constexpr uint32_t LANE_MAX_NODES = (1u << 26) - 1u;  // per graph: 26 bits of a tag
+constexpr uint32_t LANE_MAX_INDEG = 65534;  // pending predecessors in 16 bits, all ones for an exhausted stream
+constexpr uint32_t LANE_ROUNDS = 4;       // issues on the same SMs before the records are looked over again
+// A head's tag: node id within the graph << 5 | slot on the SM, so that tags order as ids do; WAITING on top for a
+// LOAD or STORE that has no HBM server yet.
+constexpr uint32_t WAITING = 0x80000000u;
+constexpr uint32_t TAG_ID = 0x7FFFFFE0u;
+// meta: pending predecessors << 16 | successors (7: look up) << 13 | type << 10 | byte offset of the SM's servers
+constexpr uint32_t EXHAUSTED = 0xFFFF0000u;
+constexpr uint32_t LANE_DEG_BIG = 7;
+
+struct LaneLayout {
+  uint32_t Scta, NS, SC, per, per4, cap_hbm;
+  uint32_t o_type, o_slot, o_scout, o_sm, o_list, o_cand, o_cta, o_sv, o_hs, words;
+};
+
+__host__ __device__ inline bool make_lane_layout(const Layout &B, LaneLayout &L) {
+  if (B.nsub || B.cap_noc || B.NS > LANE_MAX_SMS || B.per > LANE_MAX_SLOTS) return false;
+  L.Scta = B.Scta; L.NS = B.NS; L.SC = B.SC + 1; L.per = B.per; L.per4 = (B.per + 3u) & ~3u; L.cap_hbm = B.cap_hbm;
+  uint64_t w = O_DYN;
+  L.o_type = (uint32_t)w; w += 32;
+  L.o_slot = (uint32_t)w; w += (uint64_t)L.NS * L.per4 * LANE_SLOT_WORDS;
+  L.o_scout = (uint32_t)w; w += (uint64_t)L.NS * L.per4;
+  L.o_sm = (uint32_t)w; w += (uint64_t)L.NS * LANE_SM_WORDS;
+  L.o_list = (uint32_t)w; w += 64 + LANE_CHUNKS;
+  L.o_cand = (uint32_t)w; w += L.NS;
+  w = (w + 1) & ~(uint64_t)1;  // CTA records are read as 8-byte pairs
+  L.o_cta = (uint32_t)w; w += (uint64_t)L.Scta * 2;
+  L.o_sv = (uint32_t)w; w += (uint64_t)L.NS * L.SC;
+  L.o_hs = (uint32_t)w; w += L.cap_hbm;
+  w = (w + 3) & ~(uint64_t)3;
+  if (w * 4 > MAX_SMEM_BYTES) return false;
+  L.words = (uint32_t)w;
+  return true;
+}
+
+// A row whose nodes all take at least one cycle: zero_types has a bit per type
+// with a node of no work (or a NOP) and no extra latency.
+__host__ __device__ inline bool lane_row_ok(const int32_t *p, uint32_t zero_types) {
+  const int64_t base[8] = {(int64_t)p[GTS_P_TMA_LAT] + p[GTS_P_DRAM_LAT], p[GTS_P_SMEM_LAT], p[GTS_P_MMA_LAT],
+                           p[GTS_P_ALU_LAT], p[GTS_P_TMA_LAT], 1, 0, 0};
+  for (int k = 0; k < 8; k++)
+    if (((zero_types >> k) & 1u) && base[k] == 0) return false;
+  return p[GTS_P_ISSUE_POLICY] == GTS_POLICY_LOWEST_ID && p[GTS_P_L2_BYTES] == 0;
+}
+
+// Rows of one SM leave the lanes nothing to share: the one-SM pipeline study (1,536
+// rows) took 2.2 ms here and 1.97 ms in k_simulate.
+inline bool lane_pays(const Layout &L) { return L.NS >= 2; }
+
+// Estimated cost of a row, from measured points of wsgemm, FlashAttention and
+// decoder tables: cycles per node are those of a round (3,200 + 20 per simulated
+// SM, which the grants and scans grow with) over the SMs that issue in it.  x SMs
+// have work when HBM keeps up with x of them (memory time against the busiest
+// per-SM unit's); x / (1 + x / 30) issue in a round of 32 lanes (measured 7.6 for 8
+// SMs, 5.6 where HBM feeds 6.2 of 108, 21 of 70, 25 of 132).
+__host__ __device__ inline float lane_cost(const float *work, const int32_t *row, float ns, float nodes) {
+  const float mem = work[WK_MEM] / ((float)row[GTS_P_HBM_BPC] * (float)row[GTS_P_CAP_HBM]);
+  float sm = work[WK_MEM] / ((float)row[GTS_P_TMA_BPC] * (float)row[GTS_P_CAP_TMA]);
+  sm = fmaxf(sm, work[WK_SMEM] / ((float)row[GTS_P_SMEM_BPC] * (float)row[GTS_P_CAP_LSU]));
+  sm = fmaxf(sm, work[WK_FMA] / ((float)row[GTS_P_MMA_FMA_PC] * (float)row[GTS_P_CAP_TENSOR]));
+  sm = fmaxf(sm, work[WK_EW] / ((float)row[GTS_P_ALU_OPS_PC] * (float)row[GTS_P_CAP_ALU]));
+  const float x = fmaxf(1.0f, fminf(ns, mem > 0.0f ? sm / mem : ns));
+  return nodes * (3200.0f + 20.0f * ns) * (1.0f + x / 30.0f) / x;
+}
+
+// Cost classes of a batch whose dearest row costs `top`: its points are handed out
+// class by class, in the table's order inside a class, so that the dearest do not
+// start last.  One class when every point starts at once (top = 0).
+constexpr uint32_t LANE_CLASSES = 4;
+__device__ __forceinline__ uint32_t lane_class(float cost, float top) {
+  return cost > 0.55f * top ? 0u : cost > 0.4f * top ? 1u : cost > 0.3f * top ? 2u : 3u;
+}
+
+// The next design point of a warp, as next_point_of, class by class.
+__device__ __noinline__ uint32_t lane_next_point(const DevGraph *g, const int32_t *params, const uint32_t *order,
+                                                 uint32_t n_order, uint32_t *counter, uint32_t first, uint32_t n,
+                                                 float top, int lane) {
+  for (;;) {
+    uint32_t k = 0;
+    if (lane == 0) k = atomicAdd(counter, 1u);
+    k = __shfl_sync(FULL, k, 0);
+    uint32_t c = 0;
+    while (c < LANE_CLASSES && k >= n_order) {
+      k -= n_order;
+      c++;
+    }
+    if (c >= (top > 0.0f ? LANE_CLASSES : 1u)) return NONE;
+    const uint32_t pa = order[k];
+    if (pa < first || pa - first >= n) continue;
+    if (top > 0.0f) {
+      const int32_t *row = params + (size_t)pa * GTS_NPARAM;
+      const int32_t gi = row[GTS_P_GRAPH_INDEX], cps = row[GTS_P_CTAS_PER_SM];
+      uint32_t cls = LANE_CLASSES - 1u;  // rows that will be refused
+      if (gi >= 0 && (uint32_t)gi < g->G && cps >= 1) {
+        const float ctas = (float)(g->cta_off[gi + 1] - g->cta_off[gi]);
+        const float ns = fminf((float)row[GTS_P_NUM_SMS], ceilf(ctas / (float)cps));
+        cls = lane_class(lane_cost(g->work, row, ns, (float)(g->node_off[gi + 1] - g->node_off[gi])), top);
+      }
+      if (cls != c) continue;
+    }
+    return pa - first;
+  }
+}
+
+struct LanePt {
+  uint32_t *sp;
+  LaneLayout L;
+  uint32_t W, cps, n0, c0, c1;
+  int32_t *st, *fi;
+  uint2 *scr;
+  uint64_t offs;  // byte k: offset, on an SM, of the servers of type k (the last word, always 0, for NOP)
+  uint32_t caps;  // 6 bits per class
+  uint32_t off_ld, cap_tma;  // servers of LOAD and STORE
+  uint32_t mW, mCps;
+  __device__ __forceinline__ uint4 *slots(uint32_t s) const {
+    return reinterpret_cast<uint4 *>(sp + L.o_slot + s * (L.per4 * LANE_SLOT_WORDS));
+  }
+  __device__ __forceinline__ uint4 *smrec(uint32_t s) const {
+    return reinterpret_cast<uint4 *>(sp + L.o_sm + s * LANE_SM_WORDS);
+  }
+  __device__ __forceinline__ uint2 *cta(uint32_t j) const {  // nodes not issued (0: free or finished), max finish (NONE: free)
+    return reinterpret_cast<uint2 *>(sp + L.o_cta + 2 * j);
+  }
+  __device__ __forceinline__ uint32_t *scouts(uint32_t s) const { return sp + L.o_scout + s * L.per4; }
+  __device__ __forceinline__ uint32_t *servers(uint32_t s) const { return sp + L.o_sv + s * L.SC; }
+  __device__ __forceinline__ uint32_t type_off(uint32_t type) const { return (uint32_t)(offs >> (8u * type)) & 255u; }
+  __device__ __forceinline__ uint32_t type_cap(uint32_t type) const {
+    return (uint32_t)((uint64_t)caps >> (6u * ((TYPE_CLASS >> (4 * type)) & 7u))) & 63u;  // 0 for NOP
+  }
+};
+
+// An SM's servers of one class are kept ascending: a node takes the first, and its
+// next free cycle x goes where it belongs.
+__device__ __forceinline__ void take_server(uint32_t *sv, uint32_t cap, uint32_t x) {
+  if (cap <= 4u) {
+    const uint32_t v1 = cap > 1u ? sv[1] : INF, v2 = cap > 2u ? sv[2] : INF, v3 = cap > 3u ? sv[3] : INF;
+    sv[0] = min(v1, x);
+    if (cap > 1u) sv[1] = max(v1, min(v2, x));
+    if (cap > 2u) sv[2] = max(v2, min(v3, x));
+    if (cap > 3u) sv[3] = max(v3, x);
+  } else {
+    uint32_t q = 1;
+#pragma unroll 1
+    for (; q < cap && sv[q] < x; q++) sv[q - 1] = sv[q];
+    sv[q - 1] = x;
+  }
+}
+
+// One lane: SM s's record at horizon H.
+//  a: key and tag of its first head without WAITING by (key, id); max(key, H) and tag of its first waiting head by
+//     (max(key, H), id) -- H never falls, so the key itself is not needed
+//  b: first retirement of a finished CTA; the earliest cycle issuing the first head can show a new HBM head; the H
+//     from which a waiting head of lower id comes first (0: out of date); a bound below the tags of HBM heads not
+//     waiting yet
+// Slots are read four at a time without branches; an SM's slots are padded to a
+// multiple of four with exhausted streams.
+__device__ __forceinline__ void lane_refresh(const LanePt &P, uint32_t s, uint32_t H, uint4 &a, uint4 &b) {
+  const uint32_t *sv = P.servers(s);
+  const uint4 *sl = P.slots(s);
+  uint32_t kn = INF, in = NONE, eb = INF, ib = NONE, waiting = 0, nh = TAG_ID;
+  const uint32_t *sc = P.scouts(s);
+  const uint32_t F = sv[P.off_ld];
+#pragma unroll 1
+  for (uint32_t l0 = 0; l0 < P.L.per4; l0 += 4, sl += 8, sc += 4) {
+    uint4 q[4];
+    uint32_t k[4];
+    const uint4 c4 = *reinterpret_cast<const uint4 *>(sc);
+    const uint32_t c[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+    for (uint32_t u = 0; u < 4; u++) q[u] = sl[2 * u];
+#pragma unroll
+    for (uint32_t u = 0; u < 4; u++)
+      k[u] = max(q[u].x, *reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(sv) + (q[u].y & 1023u)));
+#pragma unroll
+    for (uint32_t u = 0; u < 4; u++) {
+      const bool ok = q[u].y < (1u << 16), w = (int32_t)q[u].z < 0;
+      const bool un = ok && !w && pack(k[u], q[u].z) < pack(kn, in);
+      kn = un ? k[u] : kn;
+      in = un ? q[u].z : in;
+      const uint32_t e = max(k[u], H), tag = q[u].z & ID_MASK;
+      const bool ub = ok && w && pack(e, tag) < pack(eb, ib);
+      eb = ub ? e : eb;
+      ib = ub ? tag : ib;
+      waiting += ok && w ? 1u : 0u;
+      nh = min(nh, ok && w ? TAG_ID : c[u]);
+    }
+  }
+  uint32_t k2 = INF;
+  if (waiting > 1u) {
+    sl = P.slots(s);
+#pragma unroll 1
+    for (uint32_t l = 0; l < P.L.per; l++) {
+      const uint4 q = sl[2 * l];
+      const uint32_t k = max(q.x, F);
+      if (q.y < (1u << 16) && (int32_t)q.z < 0 && (q.z & ID_MASK) < ib) k2 = min(k2, k);  // it lost: k > H
+    }
+  }
+  a = make_uint4(kn, in, eb, ib);
+  b.y = max(kn, F);
+  b.z = k2;
+  b.w = nh;
+  P.smrec(s)[0] = a;
+  P.smrec(s)[1] = b;
+}
+
+// The part of SM s's record that changes with its CTAs.
+__device__ __forceinline__ void lane_ctas(const LanePt &P, uint32_t s, uint4 &b) {
+  uint32_t U = INF;
+#pragma unroll 1
+  for (uint32_t j = s * P.cps, j1 = min(j + P.cps, P.L.Scta); j < j1; j++) {
+    const uint2 c = *P.cta(j);
+    if (!c.x) U = min(U, c.y);  // INF in a free slot
+  }
+  b.x = U;
+}
+
+// Whether SM record (a, b)'s first head may issue: before its SM's waiting HBM
+// head and not past a retirement that will launch a CTA (U).
+__device__ __forceinline__ bool lane_issuable(const uint4 &a, uint32_t H, uint32_t U) {
+  return a.x <= U && pack(a.x, a.y) < pack(max(a.z, H), a.w);
+}
+
+// ceil(n / d) given M = div_const(d), as cdiv_c, without branches.
+__device__ __forceinline__ uint32_t cdiv_flat(uint32_t n, uint32_t d, uint32_t Mlo, uint32_t Mhi) {
+  const uint64_t lo = (uint64_t)Mlo * n, hi = (uint64_t)Mhi * n + (lo >> 32);
+  const uint32_t q = (uint32_t)(hi >> 32), c = q + (q * d != n ? 1u : 0u);
+  return (Mlo | Mhi) ? c : n;
+}
+
+// Slot l of an SM (slots sl) takes node v as its head.  The type table holds rate,
+// base latency and division constant per type (rate 1 for BAR and NOP).
+__device__ __forceinline__ void lane_set_head(const LanePt &P, uint4 *sl, uint32_t l, uint32_t v, const uint4 &r,
+                                              const uint2 &se, uint32_t released, uint32_t rdy) {
+  const uint32_t type = r.w & 7u;
+  const uint4 tt = *reinterpret_cast<const uint4 *>(P.sp + P.L.o_type + 4u * type);
+  const uint32_t n = type >= GTS_BAR ? (type == GTS_BAR ? 1u : 0u) : r.x;
+  const uint32_t occ = cdiv_flat(n, tt.x, tt.z, tt.w);
+  const bool w = ((TYPE_HBM >> type) & 1u) != 0u;
+  const uint32_t hocc = cdiv_flat(n, P.sp[GTS_P_HBM_BPC], P.sp[O_MAG], P.sp[O_MAG + 1]);
+  const uint64_t lat = (uint64_t)tt.y + r.y + (w ? max(occ, hocc) : occ);
+  const uint32_t pend = (r.w >> 4) - released, deg = min(se.y - se.x, LANE_DEG_BIG);
+  sl[2 * l] = v == NONE ? make_uint4(0u, EXHAUSTED, ID_MASK, NONE)
+                        : make_uint4(rdy, pend << 16 | deg << 13 | type << 10 | P.type_off(type) << 2,
+                                     (v - P.n0) << 5 | l | (w ? WAITING : 0u), r.z);
+  sl[2 * l + 1] = make_uint4(occ, w ? hocc : P.type_cap(type), se.x, lat > 0x80000000ull ? 0x80000000u : (uint32_t)lat);
+}
+
+struct LaneState {
+  uint32_t next, nres, nrun, kernel;  // next CTA to launch; resident CTAs, those with nodes left, their kernel
+  bool blocked;                       // next's kernel waits for every resident CTA to retire
+};
+
+__device__ __forceinline__ uint2 ld_next_type(const uint4 *rec, uint32_t v) {  // next of stream, type | in-degree << 4
+  return *(reinterpret_cast<const uint2 *>(rec + v) + 1);
+}
+
+__device__ __forceinline__ uint2 ld_succ_range(const uint4 *rng, uint32_t v) {
+  return *(reinterpret_cast<const uint2 *>(rng + v) + 1);
+}
+
+// Retires what finished by cycle T and launches as many CTAs as fit at T, up to 32
+// at a time.  SMs it touches are marked out of date.
+__device__ __forceinline__ void lane_launch(const DevGraph &g, const LanePt &P, LaneState &Q, uint32_t T,
+                                            int32_t *cta_sm_row, int lane) {
+  uint32_t freed = 0;
+#pragma unroll 1
+  for (uint32_t j = lane; j < P.L.Scta; j += 32) {
+    const uint2 c = *P.cta(j);
+    if (c.x == 0u && c.y != NONE && c.y <= T) {
+      P.cta(j)->y = NONE;
+      P.smrec(div16(j, P.mCps))[1].z = 0u;
+      freed++;
+    }
+  }
+  Q.nres -= __reduce_add_sync(FULL, freed);
+  __syncwarp();
+  uint32_t *list = P.sp + P.L.o_list;
+  Q.blocked = false;
+#pragma unroll 1
+  while (Q.next < P.c1) {
+    const uint32_t kc = g.cta_kernel[Q.next];
+    if (Q.nres && kc != Q.kernel) {
+      Q.blocked = true;
+      break;
+    }
+    uint32_t b0 = 0, bal = 0;
+#pragma unroll 1
+    for (; b0 < P.L.Scta; b0 += 32) {
+      bool fr = false;
+      if (b0 + lane < P.L.Scta) {
+        const uint2 c = *P.cta(b0 + lane);
+        fr = c.x == 0u && c.y == NONE;
+      }
+      bal = __ballot_sync(FULL, fr);
+      if (bal) break;
+    }
+    if (!bal) break;
+    if (g.cta_cnt[Q.next] == 0u) {  // an empty CTA takes the lowest free slot and leaves it in the same cycle
+      if (lane == 0 && cta_sm_row) cta_sm_row[Q.next - P.c0] = (int32_t)div16(b0 + __ffs(bal) - 1, P.mCps);
+      Q.next++;
+      continue;
+    }
+    const bool fr = (bal >> lane) & 1u;
+    const uint32_t rank = __popc(bal & ((1u << lane) - 1u)), c = Q.next + rank, j = b0 + lane;
+    bool take = fr && c < P.c1;
+    uint32_t cnt = 0;
+    if (take) {
+      cnt = g.cta_cnt[c];
+      take = cnt != 0u && g.cta_kernel[c] == kc;
+    }
+    const uint32_t bad = __ballot_sync(FULL, fr && !take);
+    if (bad) take = take && (uint32_t)lane < (uint32_t)__ffs(bad) - 1u;
+    const uint32_t m = __popc(__ballot_sync(FULL, take));
+    if (take) {
+      const uint32_t s = div16(j, P.mCps);
+      *P.cta(j) = make_uint2(cnt, 0u);
+      P.smrec(s)[1].z = 0u;
+      list[rank] = j;
+      if (cta_sm_row) cta_sm_row[c - P.c0] = (int32_t)s;
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (uint32_t x = lane; x < m * P.W; x += 32) {
+      const uint32_t r = div16(x, P.mW), w = x - r * P.W, jj = list[r], s = div16(jj, P.mCps);
+      const uint32_t v = g.stream_first[(size_t)(Q.next + r) * P.W + w];
+      uint4 rc = make_uint4(0, 0, 0, 0);
+      uint2 se = make_uint2(0, 0);
+      if (v != NONE) {  // no edge enters the CTA, so nothing was released into its nodes yet
+        rc = g.rec[v];
+        se = ld_succ_range(g.rng, v);
+      }
+      const uint32_t l = (jj - s * P.cps) * P.W + w;
+      lane_set_head(P, P.slots(s), l, v, rc, se, 0u, T);
+      P.scouts(s)[l] = v == NONE ? TAG_ID : (v - P.n0) << 5;
+    }
+    __syncwarp();
+    Q.nres += m;
+    Q.nrun += m;
+    Q.kernel = kc;
+    Q.next += m;
+  }
+  __syncwarp();
+}
+
+// Issues SM s's first head (record a) at its key; the record is then out of date.
+// Returns the finish cycle, 2^31 or more on overflow (nothing is changed then).
+// The loads are started first; the server, CTA and trace updates need none of them.
+__device__ __forceinline__ uint32_t lane_issue(const DevGraph &g, const LanePt &P, uint32_t s, uint64_t pol,
+                                               const uint4 &a, bool &cta_done) {
+  const uint32_t t = a.x, l = a.y & 31u, v = a.y >> 5;
+  uint4 *sl = P.slots(s);
+  const uint4 q = sl[2 * l], z = sl[2 * l + 1];
+  const uint32_t nx = q.w;
+  const uint2 *succ = g.succ + z.z;
+  uint32_t deg = (q.y >> 13) & 7u;
+  uint2 e0 = make_uint2(NONE, 0), e1 = e0;
+  if (deg > 0u) e0 = succ[0];
+  if (deg > 1u) e1 = succ[1];
+  uint4 rn = make_uint4(0, 0, 0, 0);
+  uint2 sn = make_uint2(0, 0), cn = make_uint2(0, 0);
+  uint2 *counters = P.scr + (nx - P.n0);
+  // the stream's scout: no node from the head up to it takes an HBM server; an odd tag says that it does itself
+  uint32_t *scout = P.scouts(s) + l;
+  const uint32_t so = *scout, at = (so >> 5) + P.n0;
+  const bool ahead = so != TAG_ID && at > nx, scan = ahead && !(so & 1u);
+  uint2 sr = make_uint2(NONE, 0);
+  if (nx != NONE) {
+    rn = g.rec[nx];
+    sn = ld_succ_range(g.rng, nx);
+    cn = ld_counters_keep(counters, pol);
+    if (scan) sr = ld_next_type(g.rec, at);
+  }
+  const uint32_t f = t + z.w, off = (q.y & 1023u) >> 2;
+  if ((int32_t)f < 0) return f;
+  if (off != P.L.SC - 1u) take_server(P.servers(s) + off, (q.y & (3u << 10)) ? z.y : P.cap_tma, t + z.x);
+  if (P.st) {
+    __stcs(P.st + v, (int32_t)t);
+    __stcs(P.fi + v, (int32_t)f);
+  }
+  const uint32_t jl = P.cps > 1u ? div16(l, P.mW) : 0u, j = s * P.cps + jl;
+  const uint2 c = *P.cta(j);
+  *P.cta(j) = make_uint2(c.x - 1u, max(c.y, f));
+  cta_done = c.x == 1u;
+  // the stream's next node becomes the head before the releases, which then reach it like any other head
+  if (cn.x | cn.y) st_counters_zero_keep(counters, pol);  // read once: leave the row clean
+  lane_set_head(P, sl, l, nx, rn, sn, cn.x, max(t, cn.y));
+  // the scout goes on: by one node, to keep its distance, or by two where an HBM head waits, to gain some (the second
+  // load overlaps the releases)
+  if (!ahead) sr = make_uint2(rn.z, rn.w);
+  const bool stop = ((TYPE_HBM >> (sr.y & 7u)) & 1u) != 0u;
+  const bool second = a.z != INF && (q.y & (3u << 10)) && !stop && sr.x != NONE && !(ahead && !scan);
+  uint2 s2 = make_uint2(sr.x, 0);
+  if (second) s2 = ld_next_type(g.rec, sr.x);
+  const uint32_t n5 = P.n0 << 5;
+  sl += 2u * jl * P.W;
+  auto release = [&](const uint2 &e) {
+    const uint32_t rel = (e.y & 1u) ? t : f;
+    uint4 *ts = sl + (e.y & 254u);  // the successor's warp, two vectors per slot
+    const uint4 h = *ts;
+    if (((h.z ^ ((e.x << 5) - n5)) & TAG_ID) == 0u)
+      *reinterpret_cast<uint2 *>(ts) = make_uint2(max(h.x, rel), h.y - (1u << 16));
+    else
+      red_keep(P.scr + (e.x - P.n0), rel, pol);
+  };
+  if (deg > 0u) release(e0);
+  if (deg > 1u) release(e1);
+  if (deg > 2u) {
+    if (deg == LANE_DEG_BIG) deg = ld_succ_range(g.rng, v + P.n0).y - z.z;
+#pragma unroll 1
+    for (uint32_t k = 2; k < deg; k += 2) {
+      e0 = succ[k];
+      if (k + 1u < deg) e1 = succ[k + 1];
+      release(e0);
+      if (k + 1u < deg) release(e1);
+    }
+  }
+  {
+    const bool stop2 = ((TYPE_HBM >> (s2.y & 7u)) & 1u) != 0u;
+    const uint32_t to = stop ? (ahead ? at : nx) : (second && stop2 ? sr.x : s2.x);
+    uint32_t tag = to == NONE ? TAG_ID : (to << 5) - n5 + (stop || (second && stop2) ? 1u : 0u);
+    tag = nx == NONE || so == TAG_ID ? TAG_ID : tag;
+    *scout = ahead && !scan ? so : tag;
+  }
+  return f;
+}
+
+// HBM grants in (cycle, id) order while the first candidate precedes every bound;
+// then the task list: the granted SMs with their cycles, and those whose first head
+// H passed.  Per lane CH SMs with a waiting head in registers, each with two
+// entries: the waiting head, (max(K, H), ID) with ID its tag << 1 | 1, and the bound
+// on HBM heads its SM has not shown, (max(L, H), IM) -- (H, 0) from H >= K2 on, when
+// another waiting head comes first.  A grant leaves the bound: the next HBM head of
+// the SM waits for a TMA server.  It may precede earlier heads of its SM that use
+// other units: their issue does not depend on it, and it not on theirs.  Returns
+// the SMs granted (at most 32, one task each), NONE on overflow.
+template <uint32_t CH>
+__device__ __forceinline__ uint32_t lane_grant(const LanePt &P, uint32_t &H, bool live, int lane, uint32_t n_cand,
+                                               uint32_t min_u, uint32_t lb_h, uint32_t lb_i, uint32_t lb_2,
+                                               uint32_t lb_any, uint32_t &n_task) {
+  const uint32_t below = (1u << lane) - 1u;
+  uint32_t K[CH], ID[CH], L[CH], IM[CH], K2[CH], HO[CH], OC[CH];
+  uint32_t granted = 0, n_granted = 0;
+#pragma unroll
+  for (uint32_t c = 0; c < CH; c++) {
+    K[c] = L[c] = K2[c] = INF;
+    ID[c] = IM[c] = NONE << 1;
+    HO[c] = OC[c] = 0;
+    if (32u * c + lane < n_cand) {
+      const uint32_t s = P.sp[P.L.o_cand + 32u * c + lane];
+      const uint4 a = P.smrec(s)[0], b = P.smrec(s)[1];
+      const uint32_t U = live ? b.x : INF;
+      const uint2 o = *reinterpret_cast<const uint2 *>(P.slots(s) + 2 * (a.w & 31u) + 1);
+      K[c] = a.z;
+      ID[c] = a.w << 1 | (max(a.z, H) <= U ? 1u : 0u);
+      // a first head after the waiting one shows nothing before it, and at its own cycle only higher ids
+      L[c] = a.x == INF ? INF : lane_issuable(a, H, INF) ? b.y : a.x + (a.y > a.w ? 1u : 0u);
+      IM[c] = b.w << 1;
+      K2[c] = b.z;
+      HO[c] = o.y;
+      OC[c] = P.cap_tma == 1u ? o.x : 0u;
+    }
+  }
+#pragma unroll 1
+  while (n_granted < 32u) {
+    const uint32_t ux = max(min_u, H);
+    uint32_t x = max(lb_h, H), y = H > lb_h && H >= lb_2 ? lb_any : lb_i, at = 0;
+    if (pack(ux, 0xFFFFFFFEu) < pack(x, y)) {
+      x = ux;
+      y = 0xFFFFFFFEu;
+    }
+#pragma unroll
+    for (uint32_t c = 0; c < CH; c++) {
+      if (c == 0u || 32u * c < n_cand) {
+        const bool th = H >= K2[c];
+        const uint32_t bx = th ? H : max(L[c], H), by = th ? 0u : IM[c];
+        uint32_t cx = max(K[c], H), cy = ID[c];
+        const bool bound = pack(bx, by) < pack(cx, cy);
+        cx = bound ? bx : cx;
+        cy = bound ? by : cy;
+        const bool less = pack(cx, cy) < pack(x, y);
+        x = less ? cx : x;
+        y = less ? cy : y;
+        at = less ? c : at;
+      }
+    }
+    const uint32_t t = __reduce_min_sync(FULL, x);
+    const uint32_t first = __reduce_min_sync(FULL, x == t ? y : NONE);
+    if (!(first & 1u) || t == INF) break;
+    const bool win = x == t && y == first;
+    uint32_t ho = HO[0];
+#pragma unroll
+    for (uint32_t c = 1; c < CH; c++) ho = at == c ? HO[c] : ho;
+    ho = __reduce_max_sync(FULL, win ? ho : 0u);
+    if ((uint64_t)t + ho > 0x7FFFFFFFull) return NONE;
+    n_granted++;
+    granted |= win ? 1u << at : 0u;
+#pragma unroll
+    for (uint32_t c = 0; c < CH; c++) {
+      const bool mine = win && at == c;
+      L[c] = mine ? t + OC[c] : L[c];
+      IM[c] = mine ? (K2[c] != INF ? 0u : min(IM[c], ID[c] & ~1u)) : IM[c];  // K2: a waiting head of lower id
+      K[c] = mine ? INF : K[c];
+      K2[c] = mine ? INF : K2[c];
+      HO[c] = mine ? t : HO[c];
+    }
+    if (P.L.cap_hbm == 1u) {
+      H = t + ho;
+    } else {
+      uint32_t *hs = P.sp + P.L.o_hs;
+      const bool in = (uint32_t)lane < P.L.cap_hbm;
+      uint32_t hv = in ? hs[lane] : INF;
+      const uint32_t bal = __ballot_sync(FULL, in && hv <= t);
+      if (lane == __ffs(bal) - 1) hs[lane] = hv = t + ho;
+      H = __reduce_min_sync(FULL, hv);
+    }
+  }
+  uint32_t *listed = P.sp + P.L.o_list + 64;
+#pragma unroll
+  for (uint32_t c = 0; c < CH; c++) {
+    if (32u * c < n_cand) {
+      const bool go = (granted >> c) & 1u;
+      const uint32_t bal = __ballot_sync(FULL, go);
+      if (go) {
+        const uint32_t s = P.sp[P.L.o_cand + 32u * c + lane];
+        uint32_t *li = P.sp + P.L.o_list + n_task + __popc(bal & below);
+        li[0] = s;
+        li[32] = HO[c];
+        atomicOr(listed + (s >> 5), 1u << (s & 31u));
+      }
+      n_task += __popc(bal);
+    }
+  }
+#pragma unroll
+  for (uint32_t c = 0; c < CH; c++) {
+    if (32u * c < n_cand && n_task < 32u) {
+      const bool go = L[c] < H && !((granted >> c) & 1u);  // its first head's key is at most L (and may be past a retirement)
+      const uint32_t bal = __ballot_sync(FULL, go), at = n_task + __popc(bal & below);
+      if (go && at < 32u) {
+        const uint32_t s = P.sp[P.L.o_cand + 32u * c + lane];
+        P.sp[P.L.o_list + at] = s;
+        atomicOr(listed + (s >> 5), 1u << (s & 31u));
+      }
+      n_task += __popc(bal);
+    }
+  }
+  return n_granted;
+}
+
+__global__ void __launch_bounds__(MAX_WPB * 32, 3)
+k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__ params, uint32_t first_point, uint32_t n_points, uint32_t flags,
+                 int32_t *d_start, int32_t *d_finish, int32_t *d_makespan, int32_t *d_status, uint64_t *d_digest,
+                 int32_t *d_cta_sm, int64_t *d_busy, uint2 *scratch, uint32_t n_warps, uint32_t budget_words,
+                 const uint32_t *__restrict__ order, uint32_t n_order, float top) {
+  extern __shared__ __align__(16) uint32_t smem[];
+  const int lane = threadIdx.x & 31;
+  const uint32_t wib = threadIdx.x >> 5;
+  const uint32_t gw = blockIdx.x * (blockDim.x >> 5) + wib;
+  if (gw >= n_warps) return;
+  LanePt P;
+  uint32_t *sp = P.sp = smem + wib * budget_words;
+  P.W = g.W;
+  const bool want_digest = d_digest != nullptr;
+  bool row_clean = (flags & GTS_SCRATCH_CLEAN) != 0u;
+  const uint64_t pol = keep_policy();
+  const uint32_t below = (1u << lane) - 1u;
+  uint32_t *next_point = reinterpret_cast<uint32_t *>(scratch);
+  uint32_t q = gw;
+  for (bool begun = false;; begun = true) {
+    if (order) q = lane_next_point(&g, params, order, n_order, next_point, first_point, n_points, top, lane);
+    else q = begun ? (q + n_warps < n_points ? q + n_warps : NONE) : (gw < n_points ? gw : NONE);
+    if (q == NONE) break;
+    const uint32_t p = first_point + q;
+    if (lane < GTS_NPARAM) sp[lane] = (uint32_t)params[(size_t)p * GTS_NPARAM + lane];
+    __syncwarp();
+    const int32_t *prm = reinterpret_cast<const int32_t *>(sp);
+    int status = check_row(prm, g.G, g.class_mask);
+    const uint32_t gi = status == GTS_OK ? (uint32_t)prm[GTS_P_GRAPH_INDEX] : 0u;
+    P.n0 = g.node_off[gi];
+    const uint32_t nG = g.node_off[gi + 1] - P.n0;
+    P.c0 = g.cta_off[gi];
+    P.c1 = g.cta_off[gi + 1];
+    const uint32_t CG = P.c1 - P.c0;
+    if (status == GTS_OK) {
+      Layout B;
+      if (!make_layout(prm, CG, P.W, g.class_mask, B) || !make_lane_layout(B, P.L) || P.L.words > budget_words ||
+          !lane_row_ok(prm, g.zero_types))
+        status = GTS_ERR_UNSUPPORTED;
+    }
+    if (status != GTS_OK) {
+      if (lane == 0) {
+        d_status[q] = status;
+        d_makespan[q] = 0;
+        if (want_digest) d_digest[q] = 0;
+      }
+      if (d_busy && lane < GTS_BUSY_CLASSES) d_busy[(size_t)q * GTS_BUSY_CLASSES + lane] = 0;
+      __syncwarp();
+      continue;
+    }
+    P.cps = (uint32_t)prm[GTS_P_CTAS_PER_SM];
+    P.mW = div16_const(P.W);
+    P.mCps = div16_const(P.cps);
+    P.st = (flags & GTS_FULL_TRACE) ? d_start + (size_t)q * g.row_nodes : nullptr;
+    P.fi = (flags & GTS_FULL_TRACE) ? d_finish + (size_t)q * g.row_nodes : nullptr;
+    P.scr = scratch + GTS_SCRATCH_HEADER_BYTES / 8 + (size_t)gw * (((g.row_nodes + 1u) & ~1u) + 2u * g.n_tiles);
+    int32_t *cta_sm_row = (flags & GTS_WANT_CTA_SM) ? d_cta_sm + (size_t)q * g.row_ctas : nullptr;
+    {  // servers are kept only for the classes the graph uses; types without one read the SM's last word
+      uint32_t off = 0;
+      uint64_t by_class = 0;
+      P.caps = 0;
+      for (uint32_t r = 0; r < RC_N; r++) {
+        const uint32_t c = ((g.class_mask >> r) & 1u) ? (uint32_t)prm[GTS_P_CAP_TENSOR + r] : 0u;
+        by_class |= (uint64_t)(c ? off : P.L.SC - 1u) << (8 * r);
+        P.caps |= c << (6 * r);
+        off += c;
+      }
+      P.offs = 0;
+      for (uint32_t k = 0; k < 8; k++) {
+        const uint32_t r = (TYPE_CLASS >> (4 * k)) & 15u;
+        P.offs |= (r < RC_N ? (by_class >> (8 * r)) & 255u : (uint64_t)(P.L.SC - 1u)) << (8 * k);
+      }
+      P.off_ld = P.type_off(GTS_LOAD);
+      P.cap_tma = P.type_cap(GTS_LOAD);
+    }
+    put_constants(sp, prm, lane);
+    __syncwarp();
+    if (lane < 8) {  // type table: rate, base latency, division constant
+      const uint32_t rt = (TYPE_RATE >> (4 * lane)) & 15u;
+      const uint64_t M = rt < 5u ? *reinterpret_cast<const uint64_t *>(sp + O_MAG + 2 * rt) : 0ull;
+      *reinterpret_cast<uint4 *>(sp + P.L.o_type + 4 * lane) =
+          make_uint4(rt < 5u ? sp[GTS_P_HBM_BPC + 2 * rt] : 1u, sp[O_BASE + lane], (uint32_t)M, (uint32_t)(M >> 32));
+    }
+    for (uint32_t i = lane; i < P.L.NS * P.L.per4; i += 32) {
+      P.slots(0)[2 * i] = make_uint4(0u, EXHAUSTED, ID_MASK, NONE);
+      P.slots(0)[2 * i + 1] = make_uint4(0u, 0u, 0u, 0u);
+      P.scouts(0)[i] = TAG_ID;
+    }
+    for (uint32_t s = lane; s < P.L.NS; s += 32) {
+      P.smrec(s)[0] = make_uint4(INF, NONE, INF, NONE);
+      P.smrec(s)[1] = make_uint4(INF, INF, INF, TAG_ID);
+    }
+    for (uint32_t j = lane; j < P.L.Scta; j += 32) *P.cta(j) = make_uint2(0u, NONE);
+    for (uint32_t k = lane; k < P.L.NS * P.L.SC; k += 32) sp[P.L.o_sv + k] = 0u;
+    for (uint32_t k = lane; k < P.L.cap_hbm; k += 32) sp[P.L.o_hs + k] = 0u;
+    if (!row_clean) {
+      uint4 *z = reinterpret_cast<uint4 *>(P.scr);
+      const uint32_t nz = ((g.row_nodes + 1u) >> 1) + g.n_tiles;
+      for (uint32_t k = lane; k < nz; k += 32) z[k] = make_uint4(0, 0, 0, 0);
+      row_clean = true;
+    }
+    if (cta_sm_row)
+      for (uint32_t c = lane; c < CG; c += 32) cta_sm_row[c] = -1;
+    __threadfence();
+    __syncwarp();
+
+    LaneState Q;
+    Q.next = P.c0;
+    Q.nres = Q.nrun = Q.kernel = 0;
+    Q.blocked = false;
+    uint32_t H = 0, issued = 0, mk = 0, tlast = 0;
+    uint64_t digest = 0;
+    const uint64_t limit = (8ull + P.L.NS / 8u) * nG + 4ull * CG + 64ull;  // a step grants, issues, launches or refreshes
+    uint64_t steps = 0;
+    uint32_t T = 0;  // launch cycle (INF: no launch now)
+    for (;;) {
+      if (T != INF) lane_launch(g, P, Q, T, cta_sm_row, lane);
+      T = INF;
+      if (issued >= nG) {  // trailing CTAs without nodes launch up to the last issue's cycle
+        if (Q.next >= P.c1 || nG == 0u || ++steps > limit) break;
+        uint32_t lo = INF, hi = 0;
+        for (uint32_t j = lane; j < P.L.Scta; j += 32) {
+          const uint32_t ce = P.cta(j)->y;
+          if (ce == NONE) continue;
+          lo = min(lo, ce);
+          hi = max(hi, ce);
+        }
+        T = Q.blocked ? __reduce_max_sync(FULL, hi) : __reduce_min_sync(FULL, lo);
+        if (T > __reduce_max_sync(FULL, tlast)) break;
+        continue;
+      }
+      if (++steps > limit) { status = GTS_ERR_STEP_LIMIT; break; }
+      const bool live = Q.next < P.c1 && !Q.blocked;
+      // ---- every SM: whether its first head may issue, whether a head waits for an HBM server (a candidate), whether
+      // its record is out of date.  The bound of the lane's SMs without a waiting head is (lb_h, lb_i), then (H, lb_i)
+      // while H is below their second bound lb_2, and (H, lb_any) after
+      uint32_t n_task = 0, n_cand = 0, mask = 0, min_u = INF, min_e = INF, lb_h = INF, lb_i = NONE, lb_2 = INF, lb_any = NONE;
+#pragma unroll 1
+      for (uint32_t s = lane, c = 0; s - lane < P.L.NS; s += 32, c++) {
+        uint4 a = make_uint4(INF, NONE, INF, NONE), b = make_uint4(INF, INF, INF, NONE);
+        if (s < P.L.NS) {
+          a = P.smrec(s)[0];
+          b = P.smrec(s)[1];
+        }
+        const uint32_t U = live ? b.x : INF, e = max(a.z, H);
+        const bool iss = lane_issuable(a, H, U);
+        mask |= (iss ? 1u : 0u) << c;
+        min_u = min(min_u, U);
+        min_e = min(min_e, min(a.x, e));
+        const bool cand = a.z != INF, bounds = !cand && a.x != INF;
+        const uint32_t x = bounds ? max(b.y, H) : INF, y = bounds ? b.w : NONE;
+        const bool less = pack(x, y) < pack(lb_h, lb_i);
+        lb_2 = min(lb_2, less ? lb_h : x);
+        lb_h = less ? x : lb_h;
+        lb_i = less ? y : lb_i;
+        lb_any = min(lb_any, y);
+        const uint32_t cb = __ballot_sync(FULL, cand);
+        if (cand) sp[P.L.o_cand + n_cand + __popc(cb & below)] = s;
+        n_cand += __popc(cb);
+        const bool stale = b.z <= H;
+        const uint32_t sb = __ballot_sync(FULL, stale);
+        if (sb) {
+          const uint32_t k = n_task + __popc(sb & below);
+          if (stale && k < 32u) sp[P.L.o_list + k] = s;
+          n_task += __popc(sb);
+        }
+      }
+      if (lane < (int)LANE_CHUNKS) sp[P.L.o_list + 64 + lane] = 0u;  // SMs already in the task list
+      __syncwarp();
+      const bool refresh_only = n_task != 0u;
+      uint32_t n_granted = 0;
+      if (!refresh_only) {
+        // ---- CTA launches
+        if (Q.next < P.c1) {
+          if (live) {
+            T = __reduce_min_sync(FULL, min_u);
+            if (T != INF && __reduce_min_sync(FULL, min_e) < T) T = INF;
+          } else if (Q.nrun == 0u) {  // the kernel gate opens when the last resident CTA retires
+            T = 0;
+#pragma unroll 1
+            for (uint32_t j = lane; j < P.L.Scta; j += 32) {
+              const uint32_t end = P.cta(j)->y;
+              if (end != NONE) T = max(T, end);
+            }
+            T = __reduce_max_sync(FULL, T);
+          }
+          if (T != INF) continue;
+        }
+        lb_i <<= 1;
+        lb_any <<= 1;
+        n_granted = n_cand <= 32u ? lane_grant<1>(P, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task)
+                                  : lane_grant<LANE_CHUNKS>(P, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task);
+        if (n_granted == NONE) { status = GTS_ERR_OVERFLOW; break; }
+        __syncwarp();
+#pragma unroll 1
+        for (uint32_t s = lane, c = 0; s - lane < P.L.NS && n_task < 32u; s += 32, c++) {
+          const bool go = ((mask >> c) & 1u) && !((sp[P.L.o_list + 64 + c] >> lane) & 1u);
+          const uint32_t bal = __ballot_sync(FULL, go), at = n_task + __popc(bal & below);
+          if (go && at < 32u) sp[P.L.o_list + at] = s;
+          n_task += __popc(bal);
+        }
+        if (n_task == 0u) { status = GTS_ERR_DEADLOCK; break; }
+        __syncwarp();
+      }
+      // ---- up to 32 SMs, one per lane: issue a node, then bring the SM's record up to date
+      n_task = min(n_task, 32u);
+      bool act = (uint32_t)lane < n_task;
+      uint32_t s = 0;
+      uint4 a = make_uint4(INF, NONE, INF, NONE), b = a;
+      if (act) {
+        s = sp[P.L.o_list + lane];
+        a = P.smrec(s)[0];
+        b = P.smrec(s)[1];
+        if ((uint32_t)lane < n_granted) {  // its waiting head issues at the cycle of its grant
+          a.x = sp[P.L.o_list + 32 + lane];
+          a.y = a.w;
+        } else {
+          act = refresh_only || lane_issuable(a, H, live ? b.x : INF);
+        }
+      }
+      n_task = __popc(__ballot_sync(FULL, act));
+      uint32_t left = n_task;
+      bool over = false;
+#pragma unroll 1
+      for (uint32_t round = 0; left * 2u >= n_task && round < LANE_ROUNDS; round++) {
+        bool done = false;
+        if (act) {
+          if (!refresh_only) {
+            const uint32_t f = lane_issue(g, P, s, pol, a, done);
+            over |= (int32_t)f < 0;
+            mk = max(mk, f);
+            tlast = max(tlast, a.x);
+            if (want_digest) digest += mix64(((uint64_t)(a.y >> 5) << 32 | a.x) ^ ((uint64_t)f * 0x9E3779B97F4A7C15ull));
+          }
+          if (done || refresh_only) lane_ctas(P, s, b);
+          lane_refresh(P, s, H, a, b);
+        }
+        __syncwarp();
+        if (refresh_only) break;
+        issued += left;
+        Q.nrun -= __popc(__ballot_sync(FULL, done));
+        act = act && !over && lane_issuable(a, H, live ? b.x : INF);
+        left = __popc(__ballot_sync(FULL, act));
+        if (left == 0u) break;
+      }
+      if (__any_sync(FULL, over)) { status = GTS_ERR_OVERFLOW; break; }
+      if (status != GTS_OK) break;
+      __syncwarp();
+    }
+    if (status != GTS_OK) {  // a point that stopped early may hold counters of nodes that never became heads
+      __threadfence();
+      __syncwarp();
+      uint4 *z = reinterpret_cast<uint4 *>(P.scr);
+      for (uint32_t k = lane; k < (nG + 1u) >> 1; k += 32) z[k] = make_uint4(0, 0, 0, 0);
+    }
+    __threadfence();
+    mk = __reduce_max_sync(FULL, mk);
+    if (want_digest)
+      for (int o = 16; o > 0; o >>= 1) digest += __shfl_xor_sync(FULL, digest, o);
+    if (d_busy) {  // server-cycles do not depend on the schedule: a sum over the graph's nodes
+      uint64_t busy[6] = {0, 0, 0, 0, 0, 0};
+      if (status == GTS_OK) {
+#pragma unroll 2
+        for (uint32_t v = lane; v < nG; v += 32) {
+          const uint4 r = g.rec[P.n0 + v];
+          uint32_t occ, hocc, nocc;
+          uint64_t lat;
+          node_cost<false>(sp, r.w & 15u, r.x, r.y, occ, hocc, nocc, lat);
+          const uint32_t cls = (TYPE_CLASS >> (4 * (r.w & 15u))) & 15u;
+#pragma unroll
+          for (uint32_t k = 0; k < RC_N; k++) busy[k] += cls == k ? occ : 0u;
+          busy[5] += hocc;
+        }
+      }
+      uint64_t x = 0;
+#pragma unroll
+      for (uint32_t k = 0; k < 6; k++) {
+        for (int o = 16; o > 0; o >>= 1) busy[k] += __shfl_xor_sync(FULL, busy[k], o);
+        x = (uint32_t)lane == k ? busy[k] : x;
+      }
+      if (lane < GTS_BUSY_CLASSES) d_busy[(size_t)q * GTS_BUSY_CLASSES + lane] = (int64_t)x;
+    }
+    if (lane == 0) {
+      d_status[q] = status;
+      d_makespan[q] = status == GTS_OK ? (int32_t)mk : 0;
+      if (want_digest) d_digest[q] = status == GTS_OK ? digest : 0ull;
+    }
+    __syncwarp();
+  }
+}
+
 size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct WsLayout {
@@ -1452,10 +2347,14 @@ struct WsLayout {
 enum : uint32_t {
   GK_ROWPTR = 0, GK_TYPE, GK_WARP, GK_CTA, GK_TILE, GK_EDGE, GK_KIND, GK_KERNEL, GK_INDEG, GK_NCHECKS,
   GK_CLASS = GK_NCHECKS, GK_CROSS,
+  GK_SHAPE,  // bits 0-7: types with a zero-latency node, GS_* above
   GK_SPAN_LO = 12, GK_SPAN_HI = 13,  // one 64-bit word: 8-byte aligned (the status block is 256-byte aligned)
-  GK_WORDS = 16
+  GK_WORK = 16,                      // WK_N 64-bit words: work summed over the nodes of a rate
+  GK_WORDS = GK_WORK + 2 * 4
 };
-static_assert(GK_CROSS < GK_SPAN_LO && GK_SPAN_LO % 2 == 0 && GK_SPAN_HI == GK_SPAN_LO + 1 && GK_SPAN_HI < GK_WORDS,
+constexpr uint32_t GS_UNORDERED = 1u << 8;  // some node's CTA is below the previous node's: ids are not in CTA order
+constexpr uint32_t GS_DEEP = 1u << 9;       // a node has more than LANE_MAX_INDEG predecessors
+static_assert(GK_SHAPE < GK_SPAN_LO && GK_SPAN_LO % 2 == 0 && GK_SPAN_HI == GK_SPAN_LO + 1 && GK_SPAN_HI < GK_WORDS,
               "the span sum is an aligned 64-bit word after the other status words");
 
 bool ws_layout(uint64_t n, uint64_t m, uint64_t C, uint64_t W, uint64_t G, WsLayout &w) {
@@ -1503,7 +2402,11 @@ struct GraphIn {  // the caller's arrays (gts_graph_desc)
 __global__ void k_graph_check(GraphIn in, const uint32_t *noff, const uint32_t *coff, uint32_t *stat, uint4 *rng,
                               uint32_t *first, uint32_t *cnt, uint32_t *chi) {
   const uint32_t lane = threadIdx.x & 31u;
-  uint32_t cls_or = 0u, cross = 0u;
+  uint32_t cls_or = 0u, cross = 0u, shape = 0u;
+  __shared__ unsigned long long work[WK_N];
+  unsigned long long sum[WK_N] = {0ull, 0ull, 0ull, 0ull};
+  if (threadIdx.x < WK_N) work[threadIdx.x] = 0ull;
+  __syncthreads();
   for (uint32_t v0 = blockIdx.x * blockDim.x; v0 < in.n; v0 += gridDim.x * blockDim.x) {
     const uint32_t v = v0 + threadIdx.x;
     if (v < in.n) {
@@ -1518,7 +2421,12 @@ __global__ void k_graph_check(GraphIn in, const uint32_t *noff, const uint32_t *
         const uint32_t k = (TYPE_CLASS >> (4 * ty)) & 15u;
         if (k < RC_N) cls_or |= 1u << k;
         if (k == RC_DSM) cls_or |= (1u << RC_LSU) | CM_NOC;
+        const uint32_t wk = in.work[v], wt = (TYPE_WORK >> (4 * ty)) & 15u;
+        if (in.lx[v] == 0u && (wk == 0u || ty == GTS_NOP) && ty != GTS_BAR) shape |= 1u << ty;
+#pragma unroll
+        for (uint32_t k = 0; k < WK_N; k++) sum[k] += wt == k ? wk : 0u;
       }
+      if (v > noff[g] && c < in.cta[v - 1]) shape |= GS_UNORDERED;
       if (wp >= in.W) atomicMin(&stat[GK_WARP], v);
       const bool cta_ok = c >= c0 && c < c1;
       if (!cta_ok) atomicMin(&stat[GK_CTA], v);
@@ -1545,10 +2453,20 @@ __global__ void k_graph_check(GraphIn in, const uint32_t *noff, const uint32_t *
   }
   cls_or = __reduce_or_sync(FULL, cls_or);
   cross = __reduce_or_sync(FULL, cross);
+  shape = __reduce_or_sync(FULL, shape);
   if (lane == 0) {
+    if (shape) atomicOr(&stat[GK_SHAPE], shape);
     if (cls_or) atomicOr(&stat[GK_CLASS], cls_or);
     if (cross) atomicOr(&stat[GK_CROSS], 1u);
   }
+#pragma unroll
+  for (uint32_t k = 0; k < WK_N; k++) {
+    for (int o = 16; o > 0; o >>= 1) sum[k] += __shfl_down_sync(FULL, sum[k], o);
+    if (lane == 0 && sum[k]) atomicAdd(&work[k], sum[k]);
+  }
+  __syncthreads();
+  if (threadIdx.x < WK_N && work[threadIdx.x])
+    atomicAdd(reinterpret_cast<unsigned long long *>(stat + GK_WORK) + threadIdx.x, work[threadIdx.x]);
 }
 
 // Second pass, after every in-degree and stream head is known: in-degree
@@ -1561,6 +2479,7 @@ __global__ void k_graph_check2(GraphIn in, const uint32_t *coff, uint32_t *stat,
   const uint32_t N = max(in.n, in.C);
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
     if (i < in.n && rng[i].y > MAX_INDEG) atomicMin(&stat[GK_INDEG], i);
+    if (i < in.n && rng[i].y > LANE_MAX_INDEG) atomicOr(&stat[GK_SHAPE], GS_DEEP);
     if (i < in.C) {
       if (i > 0 && graph_of(coff, in.G, i) == graph_of(coff, in.G, i - 1) && in.kern[i] < in.kern[i - 1])
         atomicMin(&stat[GK_KERNEL], i);
@@ -1647,6 +2566,7 @@ cudaError_t d2h(std::vector<T> &dst, const T *src, size_t count, cudaStream_t s)
 
 struct gts_graph {
   uint32_t n, m, C, W, G;
+  bool lanes;  // the lane-parallel instance may run it: CTA-ordered ids, no edge between CTAs, in-degrees in 16 bits
   DevGraph dg;
   int device;
   std::vector<uint32_t> node_off, cta_off;
@@ -1660,6 +2580,8 @@ struct gts_params {
   std::vector<uint8_t> sched;   // per row: asks for a per-subpartition issue policy or the L2 model
   std::vector<double> cost;     // per row: estimated simulation cost (0 for invalid rows)
   std::vector<uint8_t> wide;    // per row: SMs of 8 or more warp slots (no split SM records)
+  std::vector<float> lcost;      // per row: estimated cost in the lane-parallel instance
+  std::vector<uint32_t> lwords;  // per row: shared words in the lane-parallel instance, 0 if it cannot run there
   const uint32_t *d_order = nullptr;  // processing order (gts_params_set_order), borrowed
 };
 
@@ -1675,8 +2597,8 @@ namespace {
 // The library's handle over a packed workspace.
 gts_status make_handle(const WsLayout &wl, char *ws, uint64_t n, uint64_t m, uint64_t C, uint64_t W, uint64_t G,
                        const std::vector<uint32_t> &noff, const std::vector<uint32_t> &coff, const uint32_t *d_kernel,
-                       uint32_t row_nodes, uint32_t row_ctas, uint32_t cross, uint32_t class_mask, uint32_t n_tiles,
-                       gts_graph **out) {
+                       uint32_t row_nodes, uint32_t row_ctas, uint32_t cross, uint32_t class_mask, uint32_t shape,
+                       uint32_t n_tiles, const uint64_t *work, gts_graph **out) {
   gts_graph *g = new (std::nothrow) gts_graph();
   if (!g) return fail(GTS_ERR_INVALID_ARG, "host allocation failed");
   g->n = (uint32_t)n; g->m = (uint32_t)m; g->C = (uint32_t)C; g->W = (uint32_t)W; g->G = (uint32_t)G;
@@ -1698,6 +2620,9 @@ gts_status make_handle(const WsLayout &wl, char *ws, uint64_t n, uint64_t m, uin
   dg.row_ctas = row_ctas;
   dg.cross_cta = cross;
   dg.class_mask = class_mask;
+  for (uint32_t k = 0; k < WK_N; k++) dg.work[k] = (float)work[k];
+  dg.zero_types = shape & 255u;
+  g->lanes = !cross && !(shape & (GS_UNORDERED | GS_DEEP)) && !(class_mask & CM_NOC) && row_nodes <= LANE_MAX_NODES;
   dg.n_tiles = n_tiles;
   *out = g;
   return GTS_OK;
@@ -1906,8 +2831,10 @@ gts_status gts_graph_create(const gts_graph_desc *d, void *stream, gts_graph **o
   zero(wl.stat, 0, wl.total - wl.stat);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "graph_create: packing");
+  uint64_t work[WK_N];
+  for (uint32_t k = 0; k < WK_N; k++) work[k] = (uint64_t)st[GK_WORK + 2 * k] | (uint64_t)st[GK_WORK + 2 * k + 1] << 32;
   return make_handle(wl, ws, n, m, C, W, G, noff, coff, d->cta_kernel, row_nodes, row_ctas, st[GK_CROSS] ? 1u : 0u,
-                     st[GK_CLASS], d->tile ? d->n_tiles : 0u, out);
+                     st[GK_CLASS], st[GK_SHAPE], d->tile ? d->n_tiles : 0u, work, out);
 }
 
 size_t gts_template_workspace_bytes(uint32_t n_templates, uint32_t n_tpl_nodes, uint32_t n_nodes, uint32_t n_edges,
@@ -1961,7 +2888,9 @@ gts_status gts_graph_create_templated(const gts_template_desc *d, void *stream, 
   // ---- contract on the templates
   if (toff[0] != 0 || toff[T] != TN) return fail(GTS_ERR_INVALID_GRAPH, "tpl_node_off must run from 0 to n_tpl_nodes");
   if (row_ptr[0] != 0 || row_ptr[TN] != TE) return fail(GTS_ERR_INVALID_GRAPH, "tpl_row_ptr must run from 0 to n_tpl_edges");
-  std::vector<uint32_t> tmask(T, 0u), tindeg(TN, 0u), tnext(TN, NONE), tfirst(T * W, NONE);
+  std::vector<uint64_t> twork(T * WK_N, 0ull);
+  uint64_t work_sum[WK_N] = {0, 0, 0, 0};
+  std::vector<uint32_t> tmask(T, 0u), tshape(T, 0u), tindeg(TN, 0u), tnext(TN, NONE), tfirst(T * W, NONE);
   for (uint64_t t = 0; t < T; t++) {
     if (toff[t + 1] < toff[t]) return fail(GTS_ERR_INVALID_GRAPH, "tpl_node_off decreases at template " + std::to_string(t));
     const uint32_t u0 = toff[t], u1 = toff[t + 1];
@@ -1972,12 +2901,15 @@ gts_status gts_graph_create_templated(const gts_template_desc *d, void *stream, 
       const uint32_t cls_v = (TYPE_CLASS >> (4 * ty[u])) & 15u;
       if (cls_v < RC_N) tmask[t] |= 1u << cls_v;
       if (cls_v == RC_DSM) tmask[t] |= (1u << RC_LSU) | CM_NOC;
+      if (lx[u] == 0u && (work[u] == 0u || ty[u] == GTS_NOP) && ty[u] != GTS_BAR) tshape[t] |= 1u << ty[u];
+      if (((TYPE_WORK >> (4 * ty[u])) & 15u) < WK_N) twork[t * WK_N + ((TYPE_WORK >> (4 * ty[u])) & 15u)] += work[u];
       for (uint32_t x = row_ptr[u]; x < row_ptr[u + 1]; x++) {
         if (col[x] <= u || col[x] >= u1)
           return fail(GTS_ERR_INVALID_GRAPH, "template edge " + std::to_string(x) + " must go forward inside its template");
         if (ek[x] > 1) return fail(GTS_ERR_INVALID_GRAPH, "bad edge kind at template edge " + std::to_string(x));
         if (++tindeg[col[x]] > MAX_INDEG)
           return fail(GTS_ERR_UNSUPPORTED, "template node " + std::to_string(col[x]) + " has more than 2^24-1 predecessors");
+        if (tindeg[col[x]] > LANE_MAX_INDEG) tshape[t] |= GS_DEEP;
       }
     }
     for (uint32_t u = u1; u-- > u0;) {  // program order of each warp stream: ascending
@@ -1989,7 +2921,7 @@ gts_status gts_graph_create_templated(const gts_template_desc *d, void *stream, 
   if (coff[0] != 0 || coff[G] != C) return fail(GTS_ERR_INVALID_GRAPH, "graph_cta_off must run from 0 to n_ctas");
   std::vector<uint32_t> cbase(C), cebase(C), noff(G + 1);
   uint64_t nb = 0, eb = 0;
-  uint32_t row_nodes = 0, row_ctas = 0, class_mask = 0;
+  uint32_t row_nodes = 0, row_ctas = 0, class_mask = 0, shape = 0;
   for (uint64_t k = 0; k < G; k++) {
     if (coff[k + 1] < coff[k]) return fail(GTS_ERR_INVALID_GRAPH, "graph_cta_off decreases at graph " + std::to_string(k));
     noff[k] = (uint32_t)nb;
@@ -2003,6 +2935,8 @@ gts_status gts_graph_create_templated(const gts_template_desc *d, void *stream, 
       nb += toff[t + 1] - toff[t];
       eb += row_ptr[toff[t + 1]] - row_ptr[toff[t]];
       class_mask |= tmask[t];
+      shape |= tshape[t];
+      for (uint32_t x = 0; x < WK_N; x++) work_sum[x] += twork[t * WK_N + x];
       if (nb > n || eb > m) return fail(GTS_ERR_INVALID_GRAPH, "templates hold more nodes or edges than n_nodes / n_edges");
     }
     row_nodes = std::max(row_nodes, (uint32_t)(nb - noff[k]));
@@ -2036,7 +2970,7 @@ gts_status gts_graph_create_templated(const gts_template_desc *d, void *stream, 
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(e, "graph_create_templated: expansion");
-  return make_handle(wl, ws, n, m, C, W, G, noff, coff, d->cta_kernel, row_nodes, row_ctas, 0u, class_mask, 0u, out);
+  return make_handle(wl, ws, n, m, C, W, G, noff, coff, d->cta_kernel, row_nodes, row_ctas, 0u, class_mask, shape, 0u, work_sum, out);
 }
 
 gts_status gts_graph_destroy(gts_graph *g) {
@@ -2063,6 +2997,8 @@ gts_status gts_params_upload(gts_graph *g, const int32_t *d_params, uint32_t n_p
   P->sched.assign(n_points, 0u);
   P->cost.assign(n_points, 0.0);
   P->wide.assign(n_points, 0);
+  P->lwords.assign(n_points, 0u);
+  P->lcost.assign(n_points, 0.0f);
   for (uint32_t p = 0; p < n_points; p++) {
     const int32_t *row = h.data() + (size_t)p * GTS_NPARAM;
     if (check_row(row, g->G, g->dg.class_mask) != GTS_OK) continue;
@@ -2072,6 +3008,11 @@ gts_status gts_params_upload(gts_graph *g, const int32_t *d_params, uint32_t n_p
     if (make_layout(row, g->cta_off[gi + 1] - g->cta_off[gi], g->W, g->dg.class_mask, L)) {
       P->words[p] = L.words;
       P->wide[p] = L.per >= 8u;
+      LaneLayout LL;
+      if (g->lanes && lane_row_ok(row, g->dg.zero_types) && make_lane_layout(L, LL) && lane_pays(L)) {
+        P->lwords[p] = LL.words;
+        P->lcost[p] = lane_cost(g->dg.work, row, (float)L.NS, (float)(g->node_off[gi + 1] - g->node_off[gi]));
+      }
       // per issue the work grows slowly with the simulated SMs; the extended model costs about 3.5x
       P->cost[p] = (double)(g->node_off[gi + 1] - g->node_off[gi]) * (743.0 + L.NS) * (P->sched[p] ? 3.5 : 1.0);
     }
@@ -2113,24 +3054,32 @@ struct Plan {
   uint32_t words, wpb, smem, blocks, warps;
   bool sched;  // launch the extended instance (issue policies, NoC, L2)
   bool split;  // plain instance with split SM records (every row's SMs have fewer than 8 slots)
+  bool lanes;  // lane-parallel instance (every valid row can run there)
+  float top;   // cost of the dearest row, 0 when every point starts at once
 };
 
 gts_status plan_launch(const gts_graph *g, const gts_params *P, uint32_t first, uint32_t np, uint32_t flags,
                        size_t scratch_bytes, bool limit_by_scratch, Plan &pl) {
   (void)flags;
-  uint32_t words = 64;
+  uint32_t words = 64, lwords = 64;
+  pl.top = 0.0f;
   pl.sched = false;
+  pl.lanes = true;
   bool wide = false;
   for (uint32_t p = first; p < first + np; p++) {
     words = std::max(words, P->words[p]);
+    lwords = std::max(lwords, P->lwords[p]);
+    pl.top = std::max(pl.top, P->lcost[p]);
+    pl.lanes = pl.lanes && (P->lwords[p] || !P->words[p]);
     pl.sched = pl.sched || P->sched[p];
     wide = wide || P->wide[p];
   }
   pl.sched = pl.sched || (g->dg.class_mask & CM_NOC) != 0u;
   pl.split = !pl.sched && !wide;
+  if (pl.lanes) words = lwords;
   const uint32_t bytes = words * 4;
   pl.words = words;
-  const void *kern = pl.sched ? (const void *)k_simulate<true, false>
+  const void *kern = pl.lanes ? (const void *)k_simulate_lanes : pl.sched ? (const void *)k_simulate<true, false>
                    : pl.split ? (const void *)k_simulate<false, true> : (const void *)k_simulate<false, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
@@ -2163,6 +3112,7 @@ gts_status plan_launch(const gts_graph *g, const gts_params *P, uint32_t first, 
     warps = std::min(warps, fit);
   }
   pl.warps = (uint32_t)std::max<uint64_t>(warps, 1);
+  if (pl.warps >= np) pl.top = 0.0f;
   pl.wpb = std::min(pl.wpb, pl.warps);
   pl.smem = pl.wpb * bytes;
   pl.blocks = (pl.warps + pl.wpb - 1) / pl.wpb;
@@ -2206,11 +3156,19 @@ gts_status gts_simulate_batch(gts_graph *g, gts_params *P, uint32_t first_point,
       if (em != cudaSuccess) return cuda_fail(em, "simulate: clear the point counter");
     }
     auto kern = pl.sched ? k_simulate<true, false> : pl.split ? k_simulate<false, true> : k_simulate<false, false>;
-    kern<<<pl.blocks, pl.wpb * 32, pl.smem, s>>>(
-        g->dg, P->d_params, first_point, n_points, flags, d_start, d_finish, d_makespan, d_status,
-        (flags & GTS_WANT_DIGEST) ? d_digest : nullptr, (flags & GTS_WANT_CTA_SM) ? d_cta_sm : nullptr,
-        (flags & GTS_WANT_BUSY) ? d_busy : nullptr, (uint2 *)d_scratch, pl.warps, pl.words, P->d_order,
-        P->d_order ? P->n_points : 0u);
+    uint64_t *dig = (flags & GTS_WANT_DIGEST) ? d_digest : nullptr;
+    int32_t *csm = (flags & GTS_WANT_CTA_SM) ? d_cta_sm : nullptr;
+    int64_t *busy = (flags & GTS_WANT_BUSY) ? d_busy : nullptr;
+    const uint32_t n_order = P->d_order ? P->n_points : 0u;
+    if (pl.lanes)
+      k_simulate_lanes<<<pl.blocks, pl.wpb * 32, pl.smem, s>>>(g->dg, P->d_params, first_point, n_points, flags, d_start,
+                                                               d_finish, d_makespan, d_status, dig, csm, busy,
+                                                               (uint2 *)d_scratch, pl.warps, pl.words, P->d_order, n_order,
+                                                               pl.top);
+    else
+      kern<<<pl.blocks, pl.wpb * 32, pl.smem, s>>>(g->dg, P->d_params, first_point, n_points, flags, d_start, d_finish,
+                                                   d_makespan, d_status, dig, csm, busy, (uint2 *)d_scratch, pl.warps,
+                                                   pl.words, P->d_order, n_order);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "simulate: launch");
   }

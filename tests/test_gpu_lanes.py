@@ -1,0 +1,149 @@
+"""The lane-parallel kernel instance (one simulated SM per lane), which the
+library launches when every valid row has the lowest-id order on at least two
+SMs and the graph's ids are in CTA order with no edge between CTAs: against the
+oracle where its tiles end (SMs per lane round, slots read four at a time, the
+inline successors, servers kept in registers up to four), and against the
+general instance, which the same rows run in when the batch also holds a row of
+one SM.  Integer results, compared bit for bit."""
+import numpy as np
+import pytest
+
+from oracle import run as oracle_run
+from paper_2607_11262_gb300 import workloads as W
+from tests import gpu_helpers as H
+from tests import tinygraphs as TG
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2607_11262_gb300 import gts
+    gts.load()
+
+
+MIXES = ((W.LOAD, W.LOAD, W.STORE, W.MMA, W.EW, W.BAR), (W.LOAD, W.BAR, W.MMA), (W.LOAD, W.STORE),
+         (W.LOAD, W.SMEM, W.MMA, W.EW, W.STORE, W.BAR, W.NOP))
+
+
+def _graph(rng, n, ctas, warps, mix, kernels=False, max_work=9, p_edge=0.2, p_issue=0.3):
+    g = TG.random_graph(rng, n, W_=warps, C=ctas, p_edge=p_edge, p_issue=p_issue, intra_cta=True, kernels=kernels,
+                        types=MIXES[mix], max_work=max_work)
+    g.work = np.maximum(g.work, 1).astype(np.uint32)
+    g.lat_extra = np.where(g.type == W.NOP, 1, g.lat_extra).astype(np.uint32)  # no zero-latency node
+    return g
+
+
+def _row(rng, sms, cps, cap_hbm=1, cap_tma=1, cap_lsu=4):
+    p = TG.small_params(rng, num_sms=sms, cps=cps)
+    for k in (W.P_DRAM_LAT, W.P_TMA_LAT, W.P_SMEM_LAT, W.P_MMA_LAT, W.P_ALU_LAT):
+        p[k] = max(1, int(p[k]))
+    p[W.P_HBM_BPC] = int(rng.choice([1, 1, 2, 8]))
+    p[W.P_TMA_BPC] = int(rng.choice([1, 3, 50]))
+    p[W.P_CAP_HBM], p[W.P_CAP_TMA], p[W.P_CAP_LSU] = cap_hbm, cap_tma, cap_lsu
+    return p
+
+
+def _check(g, rows, res):
+    for q in range(rows.shape[0]):
+        H.assert_point_equal(g, rows[q], res, q, oracle_run.simulate(g, rows[q]))
+
+
+@pytest.mark.parametrize("sms", [2, 31, 32, 33, 64, 65, 160, 161])
+def test_sm_counts(sms):
+    """Around one to five SMs per lane, and one more than a lane looks after."""
+    rng = np.random.default_rng(7000 + sms)
+    for mix in range(4):
+        g = _graph(rng, 700, 170, 2, mix, kernels=mix == 3)
+        rows = np.stack([_row(rng, sms, 1, cap_hbm=c) for c in (1, 1, 3)])
+        _check(g, rows, H.run_gpu(g, rows))
+
+
+@pytest.mark.parametrize("warps,cps", [(1, 1), (3, 1), (4, 1), (5, 1), (3, 3), (8, 4), (11, 3)])
+def test_slots_per_sm(warps, cps):
+    """1 to 33 slots per SM (a lane scans up to 32)."""
+    rng = np.random.default_rng(7100 + warps * cps)
+    g = _graph(rng, 300, 20, warps, 0, kernels=True)
+    rows = np.stack([_row(rng, s, cps) for s in (2, 3, 5)])
+    _check(g, rows, H.run_gpu(g, rows))
+
+
+@pytest.mark.parametrize("caps", [(1, 1, 1), (2, 2, 2), (4, 4, 4), (1, 5, 5), (32, 32, 32)])
+def test_server_counts(caps):
+    rng = np.random.default_rng(7200 + caps[0] * 40 + caps[1])
+    for mix in (0, 3):
+        g = _graph(rng, 260, 30, 4, mix)
+        rows = np.stack([_row(rng, int(rng.choice([2, 7, 33])), int(rng.integers(1, 3)), *caps) for _ in range(6)])
+        _check(g, rows, H.run_gpu(g, rows))
+
+
+@pytest.mark.parametrize("fan", [1, 2, 3, 6, 7, 8, 40])
+def test_successor_counts(fan):
+    """Successors kept beside the head (up to 6) and looked up (7 and more)."""
+    rng = np.random.default_rng(7300 + fan)
+    n, ctas = fan + 2, 5
+    types = [W.LOAD] + [int(x) for x in rng.choice([W.MMA, W.EW, W.SMEM, W.BAR], fan)] + [W.STORE]
+    warps = [0] + [int(x) for x in rng.integers(0, 3, fan)] + [1]
+    edges = [(0, v, int(rng.integers(0, 2))) for v in range(1, fan + 1)] + [(v, n - 1, W.DATA) for v in range(1, fan + 1)]
+    g = TG.make(n * ctas, [(c * n + u, c * n + v, k) for c in range(ctas) for u, v, k in edges], types * ctas,
+                warps * ctas, [c for c in range(ctas) for _ in range(n)], 3,
+                work=[int(x) for x in rng.integers(1, 9, n * ctas)])
+    rows = np.stack([_row(rng, s, c) for s, c in ((2, 1), (3, 2), (8, 1))])
+    _check(g, rows, H.run_gpu(g, rows))
+
+
+@pytest.mark.parametrize("seed", range(6))
+def test_agrees_with_the_general_instance(seed):
+    """Rows over all forms the rule takes, alone and beside a row of one SM."""
+    rng = np.random.default_rng(7400 + seed)
+    g = _graph(rng, 400, int(rng.integers(20, 60)), int(rng.integers(1, 7)), seed % 4, kernels=seed % 2 == 1,
+               max_work=[2, 6, 60][seed % 3], p_issue=[0.0, 0.3, 0.9][seed % 3])
+    g.lat_extra[::5] += 1
+    rows = np.stack([_row(rng, int(rng.choice([2, 5, 31, 40, 130])), int(rng.choice([1, 2, 4])),
+                          int(rng.choice([1, 1, 2, 4])), int(rng.choice([1, 1, 2, 5])), int(rng.integers(1, 9)))
+                     for _ in range(24)])
+    rows[7, W.P_TMA_BPC] = 0                    # refused
+    rows[11, W.P_DRAM_LAT] = 2**31 - 40         # overflows
+    lanes = H.run_gpu(g, rows)
+    both = H.run_gpu(g, np.concatenate([rows, _row(rng, 1, 1)[None, :]]))
+    n = rows.shape[0]
+    for k in ("status", "makespan"):
+        assert np.array_equal(lanes[k], both[k][:n]), k
+    ok = lanes["status"] == 0
+    assert ok.sum() >= n - 2
+    for k in ("start", "finish", "digest", "cta_sm", "busy"):
+        assert np.array_equal(lanes[k][ok], both[k][:n][ok]), k
+
+
+def test_empty_ctas_and_gates():
+    """Empty CTAs before, between and after the others, over three kernels."""
+    rng = np.random.default_rng(7500)
+    g = _graph(rng, 120, 12, 2, 0)
+    remap = np.array([1, 2, 4, 5, 6, 9, 10, 11, 13, 15, 16, 18], np.uint32)
+    g.cta = remap[g.cta]
+    g.cta_kernel = np.array([0] * 5 + [1] * 6 + [2] * 10, np.uint32)
+    g.cta_off = np.array([0, 21], np.uint32)
+    rows = np.stack([_row(rng, s, c) for s, c in ((2, 1), (3, 2), (30, 1))])
+    _check(g, rows, H.run_gpu(g, rows))
+
+
+def test_points_taken_by_cost_class():
+    """More points than the scratch holds rows: the classes hand out every point once."""
+    import torch
+
+    from paper_2607_11262_gb300 import gts
+    w = W.workload("wsgemm_small", points=120)
+    dg = gts.DeviceGraph(w.graph)
+    dp = gts.DeviceParams(dg, w.params)
+    row = (dg.row_nodes + 1) // 2 * 16
+    few = torch.zeros(gts.GTS_SCRATCH_HEADER_BYTES + 7 * row, dtype=torch.uint8, device="cuda")
+    full = gts.simulate(dg, dp, flags=gts.GTS_WANT_DIGEST)
+    part = gts.simulate(dg, dp, first_point=11, n_points=90, flags=gts.GTS_WANT_DIGEST | gts.GTS_SCRATCH_CLEAN,
+                        scratch=few)
+    torch.cuda.synchronize()
+    assert int(full.status.abs().sum()) == 0 and int(part.status.abs().sum()) == 0
+    assert torch.equal(full.digest[11:101], part.digest) and torch.equal(full.makespan[11:101], part.makespan)
+    assert int(torch.count_nonzero(few[gts.GTS_SCRATCH_HEADER_BYTES:])) == 0
