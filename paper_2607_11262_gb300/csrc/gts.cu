@@ -31,10 +31,7 @@
 //    minimum (one pass, two independent reductions, for SMs of <= 16 slots);
 //    when H moves, the SMs whose HBM heads it overtakes are recomputed (each
 //    lane its own SMs, or one SM at a time a slot per lane when SMs hold 8
-//    slots or more).  When every SM has fewer than 8 slots, an SM whose only
-//    issuable HBM head is one keeps that head apart in its summary and takes
-//    its effective cycle max(key, H) when the summary is read, so such SMs
-//    need no recomputation when H moves.  A release into a head of another
+//    slots or more).  A release into a head of another
 //    CTA recomputes every SM (the extended instance: the SMs it reached).
 //  * The issue itself runs in every lane on broadcast values (no divergence);
 //    only global atomics and scratch-counter reads are lane 0's.
@@ -248,7 +245,7 @@ __host__ __device__ inline bool make_layout(const int32_t *p, uint32_t CG, uint3
   L.csms = (uint32_t)p[GTS_P_CLUSTER_SMS];
   L.cap_noc = (class_mask & CM_NOC) ? (uint32_t)p[GTS_P_CAP_NOC] : 0u;
   L.o_ns = (uint32_t)w;  // NoC servers per SM group
-  if (L.cap_noc) w += (uint64_t)((L.NS + L.csms - 1) / L.csms) * L.cap_noc;
+  if (L.cap_noc) w += (uint64_t)((L.NS + L.csms - 1) / L.csms) * (L.cap_noc + 1);  // and their first free cycle
   w = (w + 3) & ~(uint64_t)3;  // 16-byte multiple
   if (w * 4 > MAX_SMEM_BYTES) return false;
   L.words = (uint32_t)w;
@@ -324,7 +321,7 @@ struct Pt {
 // Occupancies and latency of a node (Section 5.2 throughput model): per-SM
 // class, HBM and NoC occupancy; latency = base + lat_extra + the largest.
 // l2: 0 no L2 model, 1 LOAD missed, 2 LOAD hit (L2 model, Section 5.2).
-template <bool EXT>
+template <bool EXT, bool NOC>
 __device__ __forceinline__ void node_cost(const uint32_t *sp, uint32_t type, uint32_t work, uint32_t lx,
                                           uint32_t &occ, uint32_t &hocc, uint32_t &nocc, uint64_t &lat,
                                           uint32_t l2 = 0u) {
@@ -334,7 +331,7 @@ __device__ __forceinline__ void node_cost(const uint32_t *sp, uint32_t type, uin
   hocc = 0u;
   if ((TYPE_HBM >> type) & 1u) hocc = cdiv_c(work, sp[GTS_P_HBM_BPC], *reinterpret_cast<const uint64_t *>(sp + O_MAG));
   nocc = 0u;
-  if (EXT && type == GTS_DSMEM) nocc = cdiv_c(work, sp[GTS_P_NOC_BPC], *reinterpret_cast<const uint64_t *>(sp + O_MAG + 10));
+  if (NOC && type == GTS_DSMEM) nocc = cdiv_c(work, sp[GTS_P_NOC_BPC], *reinterpret_cast<const uint64_t *>(sp + O_MAG + 10));
   uint32_t base = sp[O_BASE + type];
   if (EXT && l2 != 0u && type == GTS_LOAD) {  // a hit is served by L2, a miss goes through L2 to DRAM
     if (l2 == 2u) hocc = cdiv_c(work, sp[GTS_P_L2_BPC], *reinterpret_cast<const uint64_t *>(sp + O_MAG + 12));
@@ -367,7 +364,7 @@ __device__ __forceinline__ void st_counters_zero_keep(uint2 *p, uint64_t pol) {
 }
 
 // Key of slot i computed at cycle t (>= t; INF if it cannot issue yet).
-template <bool EXT>
+template <bool NOC>
 __device__ __forceinline__ uint32_t slot_key(const Pt &P, uint32_t i, uint32_t sm, uint32_t t) {
   const uint4 e = *reinterpret_cast<const uint4 *>(P.slot(i));  // {id|HBM, rdy, meta, next}
   const uint32_t h = e.x;
@@ -376,17 +373,14 @@ __device__ __forceinline__ uint32_t slot_key(const Pt &P, uint32_t i, uint32_t s
   uint32_t k = max(e.y, t);
   const uint32_t cls = meta & 7u;
   if (cls != RC_NONE) {
-    const uint32_t sc = EXT && cls == RC_DSM ? RC_LSU : cls;
+    const uint32_t sc = NOC && cls == RC_DSM ? RC_LSU : cls;
     const uint32_t *sv = P.sp + P.L.o_sv + sm * P.L.SC + P.cls_off(sc);
     const uint32_t cap = P.cls_cap(sc);
     uint32_t a = sv[0];
     for (uint32_t q = 1; q < cap; q++) a = min(a, sv[q]);
     k = max(k, a);
-    if (EXT && cls == RC_DSM) {  // and a NoC server of the SM's group
-      const uint32_t *ns = P.sp + P.L.o_ns + div16(sm, P.mCsms) * P.L.cap_noc;
-      a = ns[0];
-      for (uint32_t q = 1; q < P.L.cap_noc; q++) a = min(a, ns[q]);
-      k = max(k, a);
+    if (NOC && cls == RC_DSM) {  // and a NoC server of the SM's group
+      k = max(k, P.sp[P.L.o_ns + div16(sm, P.mCsms) * (P.L.cap_noc + 1u) + P.L.cap_noc]);
     }
   }
   return k;
@@ -397,7 +391,7 @@ __device__ __forceinline__ uint32_t slot_key(const Pt &P, uint32_t i, uint32_t s
 // E_u = max(first cycle it may issue, least effective key of its heads); its
 // pick is the first head in policy order among those whose effective key is
 // <= E_u.  The record holds the least (E_u, id of the pick) over u.
-template <bool EXT>
+template <bool NOC>
 __device__ __forceinline__ void rescan_sm_sub(const Pt &P, uint32_t s, uint32_t t, uint32_t H) {
   const uint32_t per = P.L.per, nsub = P.L.nsub, i0 = s * per;
   const uint32_t nl = min(per, P.L.S - i0);
@@ -407,7 +401,7 @@ __device__ __forceinline__ void rescan_sm_sub(const Pt &P, uint32_t s, uint32_t 
     const uint32_t *sq = P.sub(s, u);
     uint32_t m = INF;
     for (uint32_t l = u; l < nl; l += nsub) {
-      const uint32_t k = slot_key<EXT>(P, i0 + l, s, t);
+      const uint32_t k = slot_key<NOC>(P, i0 + l, s, t);
       if (k == INF) continue;
       if (P.slot(i0 + l)[F_HID] & HBM_BIT) {
         hmin = min(hmin, k);
@@ -420,7 +414,7 @@ __device__ __forceinline__ void rescan_sm_sub(const Pt &P, uint32_t s, uint32_t 
     const uint32_t E = max(m, sq[Q_AVAIL]), last = sq[Q_LAST];
     uint64_t bp = INF64;  // (policy key << 32 | slot)
     for (uint32_t l = u; l < nl; l += nsub) {
-      const uint32_t k = slot_key<EXT>(P, i0 + l, s, t);
+      const uint32_t k = slot_key<NOC>(P, i0 + l, s, t);
       if (k == INF) continue;
       const uint32_t e = (P.slot(i0 + l)[F_HID] & HBM_BIT) ? max(k, H) : k;
       if (e > E) continue;
@@ -451,14 +445,14 @@ __device__ __forceinline__ void rescan_sm_sub(const Pt &P, uint32_t s, uint32_t 
 // Warp-parallel form of rescan_sm_sub for SMs of at most 32 slots (one slot
 // per lane): each lane keys its slot once; per scheduler one reduction gives
 // E_u and a second its pick (policy keys are distinct within a scheduler).
-template <bool EXT>
+template <bool NOC>
 __device__ __forceinline__ void rescan_sm_sub_warp(const Pt &P, uint32_t s, uint32_t t, uint32_t H, int lane) {
   const uint32_t per = P.L.per, nsub = P.L.nsub, i0 = s * per;
   const uint32_t nl = min(per, P.L.S - i0);
   const uint32_t l = (uint32_t)lane;
   uint32_t e = INF, hk = INF, id = 0, u = NONE;
   if (l < nl) {
-    const uint32_t k = slot_key<EXT>(P, i0 + l, s, t);
+    const uint32_t k = slot_key<NOC>(P, i0 + l, s, t);
     const uint32_t h = P.slot(i0 + l)[F_HID];
     id = h & ID_MASK;
     u = l - div16(l, P.mSub) * nsub;
@@ -506,11 +500,11 @@ __device__ __forceinline__ void rescan_sm_sub_warp(const Pt &P, uint32_t s, uint
 
 // Warp-parallel: the keys of SM s's heads at cycle t and the SM's summary
 // record.  All lanes call it.
-template <bool EXT>
+template <bool EXT, bool NOC>
 __device__ __forceinline__ void refresh_sm(const Pt &P, uint32_t s, uint32_t t, uint32_t H, int lane) {
   if (EXT && P.L.nsub) {
-    if (P.L.per <= 32u) rescan_sm_sub_warp<EXT>(P, s, t, H, lane);
-    else if (lane == 0) rescan_sm_sub<EXT>(P, s, t, H);
+    if (P.L.per <= 32u) rescan_sm_sub_warp<NOC>(P, s, t, H, lane);
+    else if (lane == 0) rescan_sm_sub<NOC>(P, s, t, H);
     __syncwarp();
     return;
   }
@@ -521,7 +515,7 @@ __device__ __forceinline__ void refresh_sm(const Pt &P, uint32_t s, uint32_t t, 
     const uint32_t i = base + lane;
     uint64_t val = INF64;
     if (i < i1) {
-      const uint32_t k = slot_key<EXT>(P, i, s, t);
+      const uint32_t k = slot_key<NOC>(P, i, s, t);
       const uint32_t h = P.slot(i)[F_HID];
       if (k != INF) {
         const bool hb = (h & HBM_BIT) != 0u;
@@ -552,14 +546,14 @@ __device__ __forceinline__ void refresh_sm(const Pt &P, uint32_t s, uint32_t t, 
 // one pass.  Lanes below per key SM s's slots; lane 16 + j reads the record of
 // the owner's j-th SM (owner + 32 j) unless it is s; the two minima are
 // independent reductions over the same values.
-template <bool EXT>
+template <bool EXT, bool NOC>
 __device__ __forceinline__ void refresh_sm_owner(const Pt &P, uint32_t s, uint32_t t, uint32_t H, int lane, uint64_t &b,
                                                  uint32_t &bsl) {
   const uint32_t per = P.L.per, i0 = s * per, owner = s & 31u, l = (uint32_t)lane;
   uint64_t vs = INF64, vo = INF64;
   uint32_t hk = INF, so = 0;
   if (l < per && i0 + l < P.L.S) {
-    const uint32_t k = slot_key<EXT>(P, i0 + l, s, t);
+    const uint32_t k = slot_key<NOC>(P, i0 + l, s, t);
     if (k != INF) {
       const uint32_t h = P.slot(i0 + l)[F_HID];
       const bool hb = (h & HBM_BIT) != 0u;
@@ -594,17 +588,17 @@ __device__ __forceinline__ void refresh_sm_owner(const Pt &P, uint32_t s, uint32
 }
 
 // One lane: recompute the record of SM s at cycle t and horizon H.
-template <bool EXT>
+template <bool EXT, bool NOC>
 __device__ __forceinline__ void rescan_sm_lane(const Pt &P, uint32_t s, uint32_t t, uint32_t H) {
   if (EXT && P.L.nsub) {
-    rescan_sm_sub<EXT>(P, s, t, H);
+    rescan_sm_sub<NOC>(P, s, t, H);
     return;
   }
   const uint32_t i0 = s * P.L.per, i1 = min(i0 + P.L.per, P.L.S);
   uint64_t best = INF64;
   uint32_t bsl = 0, hmin = INF;
   for (uint32_t i = i0; i < i1; i++) {
-    const uint32_t k = slot_key<EXT>(P, i, s, t);
+    const uint32_t k = slot_key<NOC>(P, i, s, t);
     if (k == INF) continue;
     const uint32_t h = P.slot(i)[F_HID];
     const bool hb = (h & HBM_BIT) != 0u;
@@ -651,193 +645,6 @@ __device__ __forceinline__ void refresh_owner(const Pt &P, uint32_t owner, int l
   if ((uint32_t)lane == owner) { b = best; bsl = slot; }
 }
 
-// ---- split SM records (plain instance, SMs of fewer than 8 slots).  An SM
-// with exactly one issuable HBM head keeps it apart from its other heads:
-// words 0-1 hold the best NON-HBM head (effective cycle, id), word 2 that
-// head's slot | the HBM head's slot << 16, word 3 the HBM head's key.  The HBM
-// head's effective cycle max(key, H) is taken where the record is read, so a
-// horizon move needs no rescan of such an SM.  Any other SM keeps the whole
-// record (best head at the horizon of its last refresh, slot | SPLIT_NONE,
-// least HBM key) and is rescanned when H passes that key.
-constexpr uint32_t SPLIT_NONE = 0xFFFF0000u;
-
-__device__ __forceinline__ void put_split_rec(const Pt &P, uint32_t s, uint64_t nh, uint32_t nhslot, uint64_t all,
-                                              uint32_t allslot, uint32_t hcnt, uint32_t hslot, uint32_t hmin) {
-  uint32_t *o = P.smrec(s);
-  const bool one = hcnt == 1u;
-  const uint64_t v = one ? nh : all;
-  o[0] = (uint32_t)v;
-  o[1] = (uint32_t)(v >> 32);
-  o[2] = (v == INF64 ? 0u : (one ? nhslot : allslot)) | (one ? hslot << 16 : SPLIT_NONE);
-  o[3] = hmin;
-}
-
-// Best (effective cycle << 32 | id) of SM s at horizon H, and its slot.
-__device__ __forceinline__ uint64_t split_sm_best(const Pt &P, uint32_t s, uint32_t H, uint32_t &slot) {
-  const uint32_t *o = P.smrec(s);
-  const uint2 a = *reinterpret_cast<const uint2 *>(o);
-  const uint2 c = *reinterpret_cast<const uint2 *>(o + 2);
-  uint64_t v = pack(a.y, a.x);
-  slot = c.x & 0xFFFFu;
-  if ((c.x >> 16) != 0xFFFFu) {
-    const uint64_t hv = pack(max(c.y, H), P.slot(c.x >> 16)[F_HID] & ID_MASK);
-    if (hv < v) {
-      v = hv;
-      slot = c.x >> 16;
-    }
-  }
-  return v;
-}
-
-// Warp-parallel refresh of SM s (all its slots in one round of lanes).
-__device__ __forceinline__ void split_refresh_sm(const Pt &P, uint32_t s, uint32_t t, uint32_t H, int lane) {
-  const uint32_t i0 = s * P.L.per, i = i0 + lane;
-  uint64_t val = INF64;
-  uint32_t hk = INF;
-  bool hf = false;
-  if (lane < (int)P.L.per && i < P.L.S) {
-    const uint32_t k = slot_key<false>(P, i, s, t);
-    const uint32_t h = P.slot(i)[F_HID];
-    if (k != INF) {
-      hf = (h & HBM_BIT) != 0u;
-      val = pack(hf ? max(k, H) : k, h & ID_MASK);
-      if (hf) hk = k;
-    }
-  }
-  const uint32_t hcnt = __popc(__ballot_sync(FULL, hf));
-  uint32_t who;
-  const uint64_t m = warp_min64(hcnt == 1u && hf ? INF64 : val, who);
-  const uint32_t hmin = __reduce_min_sync(FULL, hk);
-  if (hcnt == 1u ? hf : lane == 0) put_split_rec(P, s, m, i0 + who, m, i0 + who, hcnt, i, hmin);
-  __syncwarp();
-}
-
-// Warp-parallel, as refresh_sm_owner: SM s's record and the owner lane's best
-// (b, bsl) from two independent reductions over the same values.
-__device__ __forceinline__ void split_refresh_sm_owner(const Pt &P, uint32_t s, uint32_t t, uint32_t H, int lane,
-                                                       uint64_t &b, uint32_t &bsl) {
-  const uint32_t per = P.L.per, i0 = s * per, owner = s & 31u, l = (uint32_t)lane;
-  uint64_t vs = INF64, vo = INF64;
-  uint32_t hk = INF, so = 0;
-  bool hf = false;
-  if (l < per && i0 + l < P.L.S) {
-    const uint32_t k = slot_key<false>(P, i0 + l, s, t);
-    if (k != INF) {
-      const uint32_t h = P.slot(i0 + l)[F_HID];
-      hf = (h & HBM_BIT) != 0u;
-      vs = pack(hf ? max(k, H) : k, h & ID_MASK);
-      if (hf) hk = k;
-    }
-  } else if (l >= 16u) {
-    const uint32_t sj = owner + 32u * (l - 16u);
-    if (sj < P.L.NS && sj != s) vo = split_sm_best(P, sj, H, so);
-  }
-  const bool one = __popc(__ballot_sync(FULL, hf)) == 1u;
-  uint32_t wa, wb;
-  const uint64_t ma = warp_min64(one && hf ? INF64 : vs, wa);
-  const uint64_t mb = warp_min64(vs < vo ? vs : vo, wb);
-  const uint32_t hmin = __reduce_min_sync(FULL, hk);
-  const uint32_t sb = __shfl_sync(FULL, l < 16u ? i0 + l : so, wb);
-  if (one ? hf : lane == 0) {
-    uint32_t *o = P.smrec(s);
-    o[0] = (uint32_t)ma;
-    o[1] = (uint32_t)(ma >> 32);
-    o[2] = (ma == INF64 ? 0u : i0 + wa) | (one ? (i0 + l) << 16 : SPLIT_NONE);
-    o[3] = hmin;
-  }
-  if (l == owner) {
-    b = mb;
-    bsl = mb == INF64 ? 0u : sb;
-  }
-  __syncwarp();
-}
-
-// One lane: recompute the record of SM s at cycle t and horizon H.
-__device__ __forceinline__ void split_rescan_sm_lane(const Pt &P, uint32_t s, uint32_t t, uint32_t H) {
-  const uint32_t i0 = s * P.L.per, i1 = min(i0 + P.L.per, P.L.S);
-  uint64_t best = INF64, nbest = INF64;
-  uint32_t bsl = 0, nsl = 0, hmin = INF, hcnt = 0, hslot = 0;
-  for (uint32_t i = i0; i < i1; i++) {
-    const uint32_t k = slot_key<false>(P, i, s, t);
-    if (k == INF) continue;
-    const uint32_t h = P.slot(i)[F_HID];
-    const bool hb = (h & HBM_BIT) != 0u;
-    const uint64_t val = pack(hb ? max(k, H) : k, h & ID_MASK);
-    if (hb) {
-      hmin = min(hmin, k);
-      hcnt++;
-      hslot = i;
-    } else if (val < nbest) {
-      nbest = val;
-      nsl = i;
-    }
-    if (val < best) { best = val; bsl = i; }
-  }
-  put_split_rec(P, s, nbest, nsl, best, bsl, hcnt, hslot, hmin);
-}
-
-__device__ __forceinline__ uint64_t split_lane_best(const Pt &P, int lane, uint32_t H, uint32_t &slot) {
-  uint64_t b = INF64;
-  slot = 0;
-  for (uint32_t s = lane; s < P.L.NS; s += 32) {
-    uint32_t sl;
-    const uint64_t v = split_sm_best(P, s, H, sl);
-    if (v < b) { b = v; slot = sl; }
-  }
-  return b;
-}
-
-__device__ __forceinline__ void split_refresh_owner(const Pt &P, uint32_t owner, int lane, uint32_t H, uint64_t &b,
-                                                    uint32_t &bsl) {
-  uint64_t best = INF64;
-  uint32_t slot = 0;
-  for (uint32_t base = owner; base < P.L.NS; base += 32 * 32) {
-    const uint32_t s = base + 32u * lane;
-    uint64_t val = INF64;
-    uint32_t sl = 0;
-    if (s < P.L.NS) val = split_sm_best(P, s, H, sl);
-    uint32_t who;
-    const uint64_t m = warp_min64(val, who);
-    const uint32_t ws = __shfl_sync(FULL, sl, who);
-    if (m < best) { best = m; slot = ws; }
-  }
-  if ((uint32_t)lane == owner) { b = best; bsl = slot; }
-}
-
-// Refresh entry points of the kernel: the split forms in the instance that
-// keeps split SM records, the plain ones otherwise.
-template <bool EXT, bool SPL>
-__device__ __forceinline__ void r_sm(const Pt &P, uint32_t s, uint32_t t, uint32_t H, int lane) {
-  if constexpr (SPL) split_refresh_sm(P, s, t, H, lane); else refresh_sm<EXT>(P, s, t, H, lane);
-}
-template <bool EXT, bool SPL>
-__device__ __forceinline__ void r_sm_owner(const Pt &P, uint32_t s, uint32_t t, uint32_t H, int lane, uint64_t &b,
-                                           uint32_t &bsl) {
-  if constexpr (SPL) split_refresh_sm_owner(P, s, t, H, lane, b, bsl); else refresh_sm_owner<EXT>(P, s, t, H, lane, b, bsl);
-}
-template <bool EXT, bool SPL>
-__device__ __forceinline__ void r_rescan(const Pt &P, uint32_t s, uint32_t t, uint32_t H) {
-  if constexpr (SPL) split_rescan_sm_lane(P, s, t, H); else rescan_sm_lane<EXT>(P, s, t, H);
-}
-template <bool SPL>
-__device__ __forceinline__ uint64_t r_lane_best(const Pt &P, int lane, uint32_t H, uint32_t &slot) {
-  if constexpr (SPL) return split_lane_best(P, lane, H, slot); else return lane_best(P, lane, slot);
-}
-template <bool SPL>
-__device__ __forceinline__ void r_owner(const Pt &P, uint32_t owner, int lane, uint32_t H, uint64_t &b, uint32_t &bsl) {
-  if constexpr (SPL) split_refresh_owner(P, owner, lane, H, b, bsl); else refresh_owner(P, owner, lane, b, bsl);
-}
-// SM s's record must be rescanned once H passes its least HBM key (whole records only).
-template <bool SPL>
-__device__ __forceinline__ bool r_stale(const Pt &P, uint32_t s, uint32_t H) {
-  if constexpr (SPL) {
-    const uint2 c = *reinterpret_cast<const uint2 *>(P.smrec(s) + 2);
-    return c.y < H && (c.x >> 16) == 0xFFFFu;
-  } else {
-    return P.smrec(s)[3] < H;
-  }
-}
-
 // Slot i takes node v as its head (v == NONE: stream exhausted); adj_cnt /
 // adj_rdy are releases the caller applied directly.  Every lane writes the
 // same values.
@@ -866,7 +673,7 @@ struct Clock {
 
 // Retire finished CTAs and launch as many CTAs as fit at cycle t (Section 5.1
 // TB scheduler; kernel-boundary gate).  Returns false on step-limit.
-template <bool EXT, bool SPL>
+template <bool EXT, bool NOC>
 __device__ bool launch_ctas(const DevGraph &g, Pt &P, Clock &C, int32_t *cta_sm_row, int lane, uint64_t &b,
                             uint32_t &bsl) {
   const uint32_t t = C.t;
@@ -924,8 +731,8 @@ __device__ bool launch_ctas(const DevGraph &g, Pt &P, Clock &C, int32_t *cta_sm_
     }
     __syncwarp();
     const uint32_t s = div16(freeslot, P.mCps);
-    r_sm<EXT, SPL>(P, s, t, C.H, lane);
-    r_owner<SPL>(P, s & 31u, lane, C.H, b, bsl);
+    refresh_sm<EXT, NOC>(P, s, t, C.H, lane);
+    refresh_owner(P, s & 31u, lane, b, bsl);
     C.next_cta++;
   }
 }
@@ -1010,18 +817,14 @@ __device__ __forceinline__ void put_constants(uint32_t *sp, const int32_t *prm, 
   }
 }
 
-// EXT: the kernel instance that also runs the per-subpartition issue policies
-// and the NoC of DSMEM nodes; the host launches a plain instance when no row
-// asks for a policy and the graph has no DSMEM node.  SPL: the plain instance
-// that keeps split SM records, launched when every row's SMs have fewer than 8
-// warp slots (the record forms are described above split_sm_best); the other
-// plain instance keeps whole records only.  A warp's registers come
-// from one SM sub-partition's 16K-register file, allocated 8 per thread at a
-// time: 4 warps fit per sub-partition up to 128 registers, 3 up to 168, 2
-// above.  The plain instance is held to 128 (16 warps per SM; shared memory
-// also allows 16 on rows of 132 SMs x 3 warps), the extended one to 168 (12
-// warps per SM).
-template <bool EXT, bool SPL>
+// EXT: the instances that also run the per-subpartition issue policies and the L2
+// model; NOC: and the NoC of DSMEM nodes, apart because its code costs the others
+// 2%.  The host launches the plainest one that the rows and the graph need.  A
+// warp's registers come from one SM sub-partition's 16K-register file, allocated 8
+// per thread at a time: 4 warps fit per sub-partition up to 128 registers, 3 up to
+// 168, 2 above.  The plain instance is held to 128 (16 warps per SM), the extended
+// ones to 168 (12 warps per SM).
+template <bool EXT, bool NOC>
 __global__ void __launch_bounds__(MAX_WPB * 32, EXT ? 3 : 4)
 k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point, uint32_t n_points, uint32_t flags,
            int32_t *d_start, int32_t *d_finish, int32_t *d_makespan, int32_t *d_status, uint64_t *d_digest,
@@ -1064,7 +867,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
     const bool l2on = EXT && status == GTS_OK && prm[GTS_P_L2_BYTES] != 0;
     if (status == GTS_OK) {
       if (!make_layout(prm, CG, P.W, g.class_mask, P.L) || P.L.words > budget_words ||
-          (!EXT && (P.L.nsub || P.L.cap_noc || prm[GTS_P_L2_BYTES] != 0)) || (SPL && P.L.per >= 8u))
+          (!EXT && (P.L.nsub || prm[GTS_P_L2_BYTES] != 0)) || (!NOC && P.L.cap_noc))
         status = GTS_ERR_UNSUPPORTED;
     }
     if (status != GTS_OK) {
@@ -1081,7 +884,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
     P.mW = div16_const(P.W);
     P.mCps = div16_const(P.cps);
     P.mSub = EXT ? div16_const(P.L.nsub) : 0u;
-    P.mCsms = EXT ? div16_const(P.L.csms) : 0u;
+    P.mCsms = NOC ? div16_const(P.L.csms) : 0u;
     P.policy = (uint32_t)prm[GTS_P_ISSUE_POLICY];
     P.st = (flags & GTS_FULL_TRACE) ? d_start + (size_t)q * g.row_nodes : nullptr;
     P.fi = (flags & GTS_FULL_TRACE) ? d_finish + (size_t)q * g.row_nodes : nullptr;
@@ -1109,13 +912,13 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
     }
     for (uint32_t s = lane; s < P.L.NS; s += 32) {
       uint32_t *o = P.smrec(s);
-      o[0] = NONE; o[1] = INF; o[2] = SPL ? SPLIT_NONE : 0u; o[3] = INF;
+      o[0] = NONE; o[1] = INF; o[2] = 0u; o[3] = INF;
     }
     for (uint32_t j = lane; j < P.L.Scta; j += 32) P.cta(j)[C_ID] = NONE;
     for (uint32_t k = lane; k < P.L.NS * P.L.SC; k += 32) sp[P.L.o_sv + k] = 0u;
     for (uint32_t k = lane; k < P.L.cap_hbm; k += 32) sp[P.L.o_hs + k] = 0u;
-    if (P.L.cap_noc)
-      for (uint32_t k = lane; k < ((P.L.NS + P.L.csms - 1) / P.L.csms) * P.L.cap_noc; k += 32) sp[P.L.o_ns + k] = 0u;
+    if (NOC && P.L.cap_noc)
+      for (uint32_t k = lane; k < ((P.L.NS + P.L.csms - 1) / P.L.csms) * (P.L.cap_noc + 1u); k += 32) sp[P.L.o_ns + k] = 0u;
     for (uint32_t k = lane; k < P.L.NS * P.L.nsub; k += 32) {
       sp[P.L.o_sub + k * SUB_WORDS + Q_AVAIL] = 0u;
       sp[P.L.o_sub + k * SUB_WORDS + Q_LAST] = NONE;
@@ -1147,7 +950,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
     const uint64_t l2_cap = l2on ? (uint64_t)prm[GTS_P_L2_BYTES] : 0ull;
     uint64_t b = INF64;  // this lane's best (effective cycle << 32 | id) over its SMs
     uint32_t bsl = 0;    // ... and its slot
-    if (!launch_ctas<EXT, SPL>(g, P, C, cta_sm_row, lane, b, bsl)) status = GTS_ERR_STEP_LIMIT;
+    if (!launch_ctas<EXT, NOC>(g, P, C, cta_sm_row, lane, b, bsl)) status = GTS_ERR_STEP_LIMIT;
 
     while (status == GTS_OK && issued < nG) {
       // ---- next event: minimum of (effective cycle, node id) over all heads
@@ -1160,7 +963,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
         if (++C.steps > C.limit) { status = GTS_ERR_STEP_LIMIT; break; }
         C.t = tn;
         if (C.next_ret <= C.t) {  // a CTA retires first: launch, then choose again
-          if (!launch_ctas<EXT, SPL>(g, P, C, cta_sm_row, lane, b, bsl)) { status = GTS_ERR_STEP_LIMIT; break; }
+          if (!launch_ctas<EXT, NOC>(g, P, C, cta_sm_row, lane, b, bsl)) { status = GTS_ERR_STEP_LIMIT; break; }
           continue;
         }
         // otherwise the minimum just found is the first issue at the new cycle
@@ -1208,11 +1011,11 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
           busy += ((uint32_t)lane == GTS_BUSY_L2_HITS && hit) || ((uint32_t)lane == GTS_BUSY_L2_LOADS && mem) ? 1u : 0u;
         }
       }
-      node_cost<EXT>(sp, rv.w & 15u, rv.x, rv.y, occ, hocc, nocc, lat, l2);
+      node_cost<EXT, NOC>(sp, rv.w & 15u, rv.x, rv.y, occ, hocc, nocc, lat, l2);
       const uint64_t f64 = (uint64_t)t + lat;
       if (f64 > 0x7FFFFFFFull) { status = GTS_ERR_OVERFLOW; break; }
       const uint32_t f = (uint32_t)f64;
-      const uint32_t scls = EXT && cls == RC_DSM ? RC_LSU : cls;  // the per-SM class it takes
+      const uint32_t scls = NOC && cls == RC_DSM ? RC_LSU : cls;  // the per-SM class it takes
       busy += (uint32_t)lane == scls ? occ
             : (uint32_t)lane == GTS_BUSY_HBM ? hocc : ((uint32_t)lane == GTS_BUSY_NOC ? nocc : 0u);
       // take one free server of the node's class on its SM (lane k tests server k)
@@ -1222,13 +1025,17 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
         const uint32_t bal = __ballot_sync(FULL, fr);
         if (lane == __ffs(bal) - 1) sv[lane] = t + occ;
       }
-      bool noc_touch = false;  // a NoC server of the SM's group was taken
-      if (EXT && cls == RC_DSM) {
-        uint32_t *ns = sp + P.L.o_ns + div16(sm, P.mCsms) * P.L.cap_noc;
-        const bool fr = (uint32_t)lane < P.L.cap_noc && ns[lane] <= t;
-        const uint32_t bal = __ballot_sync(FULL, fr);
-        if (lane == __ffs(bal) - 1) ns[lane] = t + nocc;
-        noc_touch = P.L.csms > 1u;
+      bool noc_touch = false;  // the last free NoC server of the SM's group was taken
+      if (NOC && cls == RC_DSM) {
+        uint32_t *ns = sp + P.L.o_ns + div16(sm, P.mCsms) * (P.L.cap_noc + 1u);
+        uint32_t v = (uint32_t)lane < P.L.cap_noc ? ns[lane] : INF;
+        const uint32_t bal = __ballot_sync(FULL, v <= t);
+        if (lane == __ffs(bal) - 1) ns[lane] = v = t + nocc;
+        v = __reduce_min_sync(FULL, v);
+        if (lane == 0) ns[P.L.cap_noc] = v;
+        // with a server still free at t, no other head's key moved; the group's first free cycle is kept, because
+        // reading all servers per key and rekeying the group at every issue took 35% of the fused attention's time
+        noc_touch = P.L.csms > 1u && v > t;
       }
       if (EXT && P.L.nsub && lane == 0) {  // the issuing scheduler: one issue per cycle, remember the slot
         const uint32_t l = i - sm * P.L.per;
@@ -1278,8 +1085,18 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
         bool to_head = false, cross = false;
         const uint32_t wc = ew.y >> 8;
         uint32_t tcs = (mine && !to_next && wc == myc) ? cs : NONE;
-        // successors in other CTAs: find each one's CTA slot, all lanes searching together
-        uint32_t xm = g.cross_cta ? __ballot_sync(FULL, mine && !to_next && wc != myc) : 0u;
+        // successors in other CTAs: where the CTAs fit at once, each sits in the slot of its rank; else find each
+        // one's slot, all lanes searching together (searching for all of them took 8% of the random DAGs' time
+        // and of the fused attention's)
+        bool away = g.cross_cta && mine && !to_next && wc != myc;
+        if (away) {
+          const uint32_t rank = wc - P.c0;
+          if (rank < P.L.Scta && P.cta(rank)[C_ID] == wc) {
+            tcs = rank;
+            away = false;
+          }
+        }
+        uint32_t xm = __ballot_sync(FULL, away);
         while (xm) {
           const int j = __ffs(xm) - 1;
           xm &= xm - 1;
@@ -1299,10 +1116,10 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
           if (tcs != NONE) {
             uint32_t *ts = P.slot(tcs * P.W + ((ew.y >> 1) & 127u));
             if ((ts[F_HID] & ID_MASK) == ew.x) {
-              atomicSub(&ts[F_META], 256u);
               atomicMax(&ts[F_RDY], rel);
+              const uint32_t left = (atomicSub(&ts[F_META], 256u) >> 8) - 1u;
               to_head = true;
-              cross = tcs != cs;
+              cross = tcs != cs && left == 0u;  // a head that waits for more predecessors keeps its key: none
               if (EXT && cross) xs = div16(tcs, P.mCps);
             }
           }
@@ -1330,7 +1147,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
       __syncwarp();
       // ---- refresh keys and summaries the issue may have changed
       if (EXT && cross_touch && deg <= 32u) {  // releases reached heads of other CTAs: their SMs and this one
-        r_sm<EXT, SPL>(P, sm, t, C.H, lane);
+        refresh_sm<EXT, NOC>(P, sm, t, C.H, lane);
         bool own = (uint32_t)lane == (sm & 31u);
         uint32_t xm = __ballot_sync(FULL, xs != NONE && xs != sm);
         uint32_t done = sm;
@@ -1340,97 +1157,84 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
           const uint32_t s2 = __shfl_sync(FULL, xs, j);
           if (s2 == done) continue;
           done = s2;
-          r_sm<EXT, SPL>(P, s2, t, C.H, lane);
+          refresh_sm<EXT, NOC>(P, s2, t, C.H, lane);
           own |= (uint32_t)lane == (s2 & 31u);
         }
         if (C.H != prevH) {  // and the SMs whose HBM heads the new horizon overtakes
           for (uint32_t s = lane; s < P.L.NS; s += 32) {
-            if (r_stale<SPL>(P, s, C.H)) {
-              r_rescan<EXT, SPL>(P, s, t, C.H);
+            if (P.smrec(s)[3] < C.H) {
+              rescan_sm_lane<EXT, NOC>(P, s, t, C.H);
               own = true;
             }
           }
         }
-        if (EXT && noc_touch) {  // the group's other SMs may hold DSMEM heads keyed on that server
+        if (NOC && noc_touch) {  // the group's other SMs may hold DSMEM heads keyed on that server
           const uint32_t g0 = div16(sm, P.mCsms) * P.L.csms, g1 = min(g0 + P.L.csms, P.L.NS);
-          for (uint32_t s = g0 + lane; s < g1; s += 32) r_rescan<EXT, SPL>(P, s, t, C.H);
+          for (uint32_t s = g0 + lane; s < g1; s += 32) rescan_sm_lane<EXT, NOC>(P, s, t, C.H);
           __syncwarp();
           for (uint32_t s = g0; s < g1; s++) own |= (s & 31u) == (uint32_t)lane;
         }
         __syncwarp();
-        if (own) b = r_lane_best<SPL>(P, lane, C.H, bsl);
+        if (own) b = lane_best(P, lane, bsl);
       } else if (cross_touch) {  // a node with many successors: recompute everything
-        for (uint32_t s = lane; s < P.L.NS; s += 32) r_rescan<EXT, SPL>(P, s, t, C.H);
+        for (uint32_t s = lane; s < P.L.NS; s += 32) rescan_sm_lane<EXT, NOC>(P, s, t, C.H);
         __syncwarp();
-        b = r_lane_best<SPL>(P, lane, C.H, bsl);
-      } else if (C.H == prevH && (SPL || P.L.per <= 16u) && P.L.NS <= 512u && !(EXT && P.L.nsub)) {
-        r_sm_owner<EXT, SPL>(P, sm, t, C.H, lane, b, bsl);
-        if (EXT && noc_touch) {  // the group's other SMs may hold DSMEM heads keyed on that server
+        b = lane_best(P, lane, bsl);
+      } else if ((C.H == prevH || P.L.NS == 1u) && P.L.per <= 16u && P.L.NS <= 512u && !(EXT && P.L.nsub)) {
+        // no other SM's record moves
+        refresh_sm_owner<EXT, NOC>(P, sm, t, C.H, lane, b, bsl);
+        if (NOC && noc_touch) {  // the group's other SMs may hold DSMEM heads keyed on that server
           const uint32_t g0 = div16(sm, P.mCsms) * P.L.csms, g1 = min(g0 + P.L.csms, P.L.NS);
           for (uint32_t s = g0 + lane; s < g1; s += 32)
-            if (s != sm) r_rescan<EXT, SPL>(P, s, t, C.H);
+            if (s != sm) rescan_sm_lane<EXT, NOC>(P, s, t, C.H);
           __syncwarp();
           bool mine = false;
           for (uint32_t s = g0; s < g1; s++) mine |= s != sm && (s & 31u) == (uint32_t)lane;
-          if (mine) b = r_lane_best<SPL>(P, lane, C.H, bsl);
+          if (mine) b = lane_best(P, lane, bsl);
         }
       } else {
-        r_sm<EXT, SPL>(P, sm, t, C.H, lane);
-        if (!SPL && C.H != prevH && P.L.per >= 8u && !(EXT && P.L.nsub)) {
+        refresh_sm<EXT, NOC>(P, sm, t, C.H, lane);
+        if (C.H != prevH && P.L.per >= 8u && !(EXT && P.L.nsub)) {
           // SMs of many slots: one SM at a time, a slot per lane
           bool own = (uint32_t)lane == (sm & 31u);
           for (uint32_t s0 = 0; s0 < P.L.NS; s0 += 32) {
             const uint32_t s = s0 + lane;
-            uint32_t xm = __ballot_sync(FULL, s < P.L.NS && s != sm && r_stale<SPL>(P, s, C.H));
+            uint32_t xm = __ballot_sync(FULL, s < P.L.NS && s != sm && P.smrec(s)[3] < C.H);
             while (xm) {
               const uint32_t s2 = s0 + __ffs(xm) - 1;
               xm &= xm - 1;
-              r_sm<EXT, SPL>(P, s2, t, C.H, lane);
+              refresh_sm<EXT, NOC>(P, s2, t, C.H, lane);
               own |= (uint32_t)lane == (s2 & 31u);
             }
           }
-          if (own) b = r_lane_best<SPL>(P, lane, C.H, bsl);
-        } else if (SPL && C.H != prevH) {
-          // split records: one pass per lane rescans its whole records that H
-          // overtook and takes its best at the new H from every record it owns
-          uint64_t nb = INF64;
-          uint32_t ns = 0;
-          for (uint32_t s = lane; s < P.L.NS; s += 32) {
-            if (s != sm && r_stale<SPL>(P, s, C.H)) r_rescan<EXT, SPL>(P, s, t, C.H);
-            uint32_t sl;
-            const uint64_t v = split_sm_best(P, s, C.H, sl);
-            if (v < nb) { nb = v; ns = sl; }
-          }
-          b = nb;
-          bsl = ns;
+          if (own) b = lane_best(P, lane, bsl);
         } else if (C.H != prevH) {
           // SMs whose HBM heads H overtakes change their effective cycles
           bool any = false;
           for (uint32_t s = lane; s < P.L.NS; s += 32) {
-            if (s != sm && r_stale<SPL>(P, s, C.H)) {
-              r_rescan<EXT, SPL>(P, s, t, C.H);
+            if (s != sm && P.smrec(s)[3] < C.H) {
+              rescan_sm_lane<EXT, NOC>(P, s, t, C.H);
               any = true;
             }
           }
-          // split records take the new H where they are read: every lane's best may move
-          if (SPL || any || (uint32_t)lane == (sm & 31u)) b = r_lane_best<SPL>(P, lane, C.H, bsl);
+          if (any || (uint32_t)lane == (sm & 31u)) b = lane_best(P, lane, bsl);
         } else {
-          r_owner<SPL>(P, sm & 31u, lane, C.H, b, bsl);
+          refresh_owner(P, sm & 31u, lane, b, bsl);
         }
-        if (EXT && noc_touch) {  // the group's other SMs may hold DSMEM heads keyed on that server
+        if (NOC && noc_touch) {  // the group's other SMs may hold DSMEM heads keyed on that server
           const uint32_t g0 = div16(sm, P.mCsms) * P.L.csms, g1 = min(g0 + P.L.csms, P.L.NS);
           for (uint32_t s = g0 + lane; s < g1; s += 32)
-            if (s != sm) r_rescan<EXT, SPL>(P, s, t, C.H);
+            if (s != sm) rescan_sm_lane<EXT, NOC>(P, s, t, C.H);
           __syncwarp();
           bool mine = false;  // this lane owns one of them
           for (uint32_t s = g0; s < g1; s++) mine |= s != sm && (s & 31u) == (uint32_t)lane;
-          if (mine) b = r_lane_best<SPL>(P, lane, C.H, bsl);
+          if (mine) b = lane_best(P, lane, bsl);
         }
       }
       __syncwarp();
       if (rem == 0u) {
         if (cend <= t) {
-          if (!launch_ctas<EXT, SPL>(g, P, C, cta_sm_row, lane, b, bsl)) { status = GTS_ERR_STEP_LIMIT; break; }
+          if (!launch_ctas<EXT, NOC>(g, P, C, cta_sm_row, lane, b, bsl)) { status = GTS_ERR_STEP_LIMIT; break; }
         } else {
           C.next_ret = min(C.next_ret, cend);
         }
@@ -2312,7 +2116,7 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
           const uint4 r = g.rec[P.n0 + v];
           uint32_t occ, hocc, nocc;
           uint64_t lat;
-          node_cost<false>(sp, r.w & 15u, r.x, r.y, occ, hocc, nocc, lat);
+          node_cost<false, false>(sp, r.w & 15u, r.x, r.y, occ, hocc, nocc, lat);
           const uint32_t cls = (TYPE_CLASS >> (4 * (r.w & 15u))) & 15u;
 #pragma unroll
           for (uint32_t k = 0; k < RC_N; k++) busy[k] += cls == k ? occ : 0u;
@@ -2579,7 +2383,6 @@ struct gts_params {
   std::vector<uint32_t> words;  // per row: shared words, 0 if the row is invalid or too large
   std::vector<uint8_t> sched;   // per row: asks for a per-subpartition issue policy or the L2 model
   std::vector<double> cost;     // per row: estimated simulation cost (0 for invalid rows)
-  std::vector<uint8_t> wide;    // per row: SMs of 8 or more warp slots (no split SM records)
   std::vector<float> lcost;      // per row: estimated cost in the lane-parallel instance
   std::vector<uint32_t> lwords;  // per row: shared words in the lane-parallel instance, 0 if it cannot run there
   const uint32_t *d_order = nullptr;  // processing order (gts_params_set_order), borrowed
@@ -2996,7 +2799,6 @@ gts_status gts_params_upload(gts_graph *g, const int32_t *d_params, uint32_t n_p
   P->words.assign(n_points, 0u);
   P->sched.assign(n_points, 0u);
   P->cost.assign(n_points, 0.0);
-  P->wide.assign(n_points, 0);
   P->lwords.assign(n_points, 0u);
   P->lcost.assign(n_points, 0.0f);
   for (uint32_t p = 0; p < n_points; p++) {
@@ -3007,7 +2809,6 @@ gts_status gts_params_upload(gts_graph *g, const int32_t *d_params, uint32_t n_p
     Layout L;
     if (make_layout(row, g->cta_off[gi + 1] - g->cta_off[gi], g->W, g->dg.class_mask, L)) {
       P->words[p] = L.words;
-      P->wide[p] = L.per >= 8u;
       LaneLayout LL;
       if (g->lanes && lane_row_ok(row, g->dg.zero_types) && make_lane_layout(L, LL) && lane_pays(L)) {
         P->lwords[p] = LL.words;
@@ -3053,7 +2854,7 @@ uint64_t scratch_row_bytes(const gts_graph *g) {
 struct Plan {
   uint32_t words, wpb, smem, blocks, warps;
   bool sched;  // launch the extended instance (issue policies, NoC, L2)
-  bool split;  // plain instance with split SM records (every row's SMs have fewer than 8 slots)
+  bool noc;    // ... with the NoC of DSMEM nodes
   bool lanes;  // lane-parallel instance (every valid row can run there)
   float top;   // cost of the dearest row, 0 when every point starts at once
 };
@@ -3065,22 +2866,19 @@ gts_status plan_launch(const gts_graph *g, const gts_params *P, uint32_t first, 
   pl.top = 0.0f;
   pl.sched = false;
   pl.lanes = true;
-  bool wide = false;
   for (uint32_t p = first; p < first + np; p++) {
     words = std::max(words, P->words[p]);
     lwords = std::max(lwords, P->lwords[p]);
     pl.top = std::max(pl.top, P->lcost[p]);
     pl.lanes = pl.lanes && (P->lwords[p] || !P->words[p]);
     pl.sched = pl.sched || P->sched[p];
-    wide = wide || P->wide[p];
   }
-  pl.sched = pl.sched || (g->dg.class_mask & CM_NOC) != 0u;
-  pl.split = !pl.sched && !wide;
+  pl.noc = (g->dg.class_mask & CM_NOC) != 0u;
   if (pl.lanes) words = lwords;
   const uint32_t bytes = words * 4;
   pl.words = words;
-  const void *kern = pl.lanes ? (const void *)k_simulate_lanes : pl.sched ? (const void *)k_simulate<true, false>
-                   : pl.split ? (const void *)k_simulate<false, true> : (const void *)k_simulate<false, false>;
+  const void *kern = pl.lanes ? (const void *)k_simulate_lanes : pl.noc ? (const void *)k_simulate<true, true>
+                   : pl.sched ? (const void *)k_simulate<true, false> : (const void *)k_simulate<false, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   int dev = 0, sms = 0;
@@ -3155,7 +2953,7 @@ gts_status gts_simulate_batch(gts_graph *g, gts_params *P, uint32_t first_point,
       const cudaError_t em = cudaMemsetAsync(d_scratch, 0, GTS_SCRATCH_HEADER_BYTES, s);
       if (em != cudaSuccess) return cuda_fail(em, "simulate: clear the point counter");
     }
-    auto kern = pl.sched ? k_simulate<true, false> : pl.split ? k_simulate<false, true> : k_simulate<false, false>;
+    auto kern = pl.noc ? k_simulate<true, true> : pl.sched ? k_simulate<true, false> : k_simulate<false, false>;
     uint64_t *dig = (flags & GTS_WANT_DIGEST) ? d_digest : nullptr;
     int32_t *csm = (flags & GTS_WANT_CTA_SM) ? d_cta_sm : nullptr;
     int64_t *busy = (flags & GTS_WANT_BUSY) ? d_busy : nullptr;
