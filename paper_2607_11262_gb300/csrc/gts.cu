@@ -1302,7 +1302,12 @@ constexpr uint32_t LANE_MAX_SMS = 32 * LANE_CHUNKS;
 constexpr uint32_t LANE_MAX_SLOTS = 32;   // warp slots per SM: five bits of a tag
 constexpr uint32_t LANE_MAX_NODES = (1u << 26) - 1u;  // per graph: 26 bits of a tag
 constexpr uint32_t LANE_MAX_INDEG = 65534;  // pending predecessors in 16 bits, all ones for an exhausted stream
-constexpr uint32_t LANE_ROUNDS = 4;       // issues on the same SMs before the records are looked over again
+// Issues on the same SMs before the records are looked over again, while two thirds
+// of them can go on.  Longer spells leave lanes idle and HBM-bound rows a round
+// behind: 4 rounds down to a half, 3 to two thirds, 3 to three quarters, 8 to a half
+// took 72.3, 67.0, 67.1, 77.5 ms on a wide ws GEMM table, 24.6, 22.7, 20.7, 29.8 on
+// attention and 31.4, 31.8, 33.2, 30.1 on a decoder layer.
+constexpr uint32_t LANE_ROUNDS = 3;
 // A head's tag: node id within the graph << 5 | slot on the SM, so that tags order as ids do; WAITING on top for a
 // LOAD or STORE that has no HBM server yet.
 constexpr uint32_t WAITING = 0x80000000u;
@@ -1316,13 +1321,16 @@ struct LaneLayout {
   uint32_t o_type, o_slot, o_scout, o_sm, o_list, o_cand, o_cta, o_sv, o_hs, words;
 };
 
-__host__ __device__ inline bool make_lane_layout(const Layout &B, LaneLayout &L) {
+// With `pad`, an SM's slots fill up to a multiple of four with exhausted streams
+// and are read as they lie; without, the last group of four repeats a slot.
+__host__ __device__ inline bool make_lane_layout(const Layout &B, bool pad, LaneLayout &L) {
   if (B.nsub || B.cap_noc || B.NS > LANE_MAX_SMS || B.per > LANE_MAX_SLOTS) return false;
-  L.Scta = B.Scta; L.NS = B.NS; L.SC = B.SC + 1; L.per = B.per; L.per4 = (B.per + 3u) & ~3u; L.cap_hbm = B.cap_hbm;
+  L.Scta = B.Scta; L.NS = B.NS; L.SC = B.SC + 1; L.per = B.per; L.per4 = pad ? (B.per + 3u) & ~3u : B.per; L.cap_hbm = B.cap_hbm;
   uint64_t w = O_DYN;
   L.o_type = (uint32_t)w; w += 32;
   L.o_slot = (uint32_t)w; w += (uint64_t)L.NS * L.per4 * LANE_SLOT_WORDS;
   L.o_scout = (uint32_t)w; w += (uint64_t)L.NS * L.per4;
+  w = (w + 3) & ~(uint64_t)3;  // SM records are read as 16-byte vectors
   L.o_sm = (uint32_t)w; w += (uint64_t)L.NS * LANE_SM_WORDS;
   L.o_list = (uint32_t)w; w += 64 + LANE_CHUNKS;
   L.o_cand = (uint32_t)w; w += L.NS;
@@ -1455,8 +1463,7 @@ __device__ __forceinline__ void take_server(uint32_t *sv, uint32_t cap, uint32_t
 //  b: first retirement of a finished CTA; the earliest cycle issuing the first head can show a new HBM head; the H
 //     from which a waiting head of lower id comes first (0: out of date); a bound below the tags of HBM heads not
 //     waiting yet
-// Slots are read four at a time without branches; an SM's slots are padded to a
-// multiple of four with exhausted streams.
+// Slots are read four at a time without branches.
 __device__ __forceinline__ void lane_refresh(const LanePt &P, uint32_t s, uint32_t H, uint4 &a, uint4 &b) {
   const uint32_t *sv = P.servers(s);
   const uint4 *sl = P.slots(s);
@@ -1464,13 +1471,29 @@ __device__ __forceinline__ void lane_refresh(const LanePt &P, uint32_t s, uint32
   const uint32_t *sc = P.scouts(s);
   const uint32_t F = sv[P.off_ld];
 #pragma unroll 1
-  for (uint32_t l0 = 0; l0 < P.L.per4; l0 += 4, sl += 8, sc += 4) {
+  for (uint32_t l0 = 0; l0 < P.L.per; l0 += 4, sl += 8, sc += 4) {
     uint4 q[4];
     uint32_t k[4];
-    const uint4 c4 = *reinterpret_cast<const uint4 *>(sc);
-    const uint32_t c[4] = {c4.x, c4.y, c4.z, c4.w};
+    uint32_t c[4];
+    if ((P.L.per4 & 3u) == 0u) {
+      const uint4 c4 = *reinterpret_cast<const uint4 *>(sc);
+      c[0] = c4.x, c[1] = c4.y, c[2] = c4.z, c[3] = c4.w;
+    } else {
+      const uint32_t last = P.L.per - 1u - l0;
 #pragma unroll
-    for (uint32_t u = 0; u < 4; u++) q[u] = sl[2 * u];
+      for (uint32_t u = 0; u < 4; u++) c[u] = sc[min(u, last)];
+    }
+    if ((P.L.per4 & 3u) == 0u) {
+#pragma unroll
+      for (uint32_t u = 0; u < 4; u++) q[u] = sl[2 * u];
+    } else {
+      const uint32_t last = P.L.per - 1u - l0;
+#pragma unroll
+      for (uint32_t u = 0; u < 4; u++) {
+        q[u] = sl[2 * min(u, last)];
+        q[u].y = u > last ? EXHAUSTED : q[u].y;
+      }
+    }
 #pragma unroll
     for (uint32_t u = 0; u < 4; u++)
       k[u] = max(q[u].x, *reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(sv) + (q[u].y & 1023u)));
@@ -1853,7 +1876,7 @@ __global__ void __launch_bounds__(MAX_WPB * 32, 3)
 k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__ params, uint32_t first_point, uint32_t n_points, uint32_t flags,
                  int32_t *d_start, int32_t *d_finish, int32_t *d_makespan, int32_t *d_status, uint64_t *d_digest,
                  int32_t *d_cta_sm, int64_t *d_busy, uint2 *scratch, uint32_t n_warps, uint32_t budget_words,
-                 const uint32_t *__restrict__ order, uint32_t n_order, float top) {
+                 const uint32_t *__restrict__ order, uint32_t n_order, float top, bool pad) {
   extern __shared__ __align__(16) uint32_t smem[];
   const int lane = threadIdx.x & 31;
   const uint32_t wib = threadIdx.x >> 5;
@@ -1885,7 +1908,7 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
     const uint32_t CG = P.c1 - P.c0;
     if (status == GTS_OK) {
       Layout B;
-      if (!make_layout(prm, CG, P.W, g.class_mask, B) || !make_lane_layout(B, P.L) || P.L.words > budget_words ||
+      if (!make_layout(prm, CG, P.W, g.class_mask, B) || !make_lane_layout(B, pad, P.L) || P.L.words > budget_words ||
           !lane_row_ok(prm, g.zero_types))
         status = GTS_ERR_UNSUPPORTED;
     }
@@ -2039,8 +2062,10 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
         }
         lb_i <<= 1;
         lb_any <<= 1;
-        n_granted = n_cand <= 32u ? lane_grant<1>(P, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task)
-                                  : lane_grant<LANE_CHUNKS>(P, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task);
+        // (two candidates per lane apart: 65.2 for 67.2 ms on the wide ws GEMM table)
+        n_granted = n_cand <= 32u   ? lane_grant<1>(P, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task)
+                    : n_cand <= 64u ? lane_grant<2>(P, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task)
+                                    : lane_grant<LANE_CHUNKS>(P, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task);
         if (n_granted == NONE) { status = GTS_ERR_OVERFLOW; break; }
         __syncwarp();
 #pragma unroll 1
@@ -2073,7 +2098,7 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
       uint32_t left = n_task;
       bool over = false;
 #pragma unroll 1
-      for (uint32_t round = 0; left * 2u >= n_task && round < LANE_ROUNDS; round++) {
+      for (uint32_t round = 0; left * 3u >= 2u * n_task && round < LANE_ROUNDS; round++) {
         bool done = false;
         if (act) {
           if (!refresh_only) {
@@ -2385,6 +2410,7 @@ struct gts_params {
   std::vector<double> cost;     // per row: estimated simulation cost (0 for invalid rows)
   std::vector<float> lcost;      // per row: estimated cost in the lane-parallel instance
   std::vector<uint32_t> lwords;  // per row: shared words in the lane-parallel instance, 0 if it cannot run there
+  std::vector<uint32_t> ltight;  // ... without padded slots
   const uint32_t *d_order = nullptr;  // processing order (gts_params_set_order), borrowed
 };
 
@@ -2800,6 +2826,7 @@ gts_status gts_params_upload(gts_graph *g, const int32_t *d_params, uint32_t n_p
   P->sched.assign(n_points, 0u);
   P->cost.assign(n_points, 0.0);
   P->lwords.assign(n_points, 0u);
+  P->ltight.assign(n_points, 0u);
   P->lcost.assign(n_points, 0.0f);
   for (uint32_t p = 0; p < n_points; p++) {
     const int32_t *row = h.data() + (size_t)p * GTS_NPARAM;
@@ -2810,8 +2837,10 @@ gts_status gts_params_upload(gts_graph *g, const int32_t *d_params, uint32_t n_p
     if (make_layout(row, g->cta_off[gi + 1] - g->cta_off[gi], g->W, g->dg.class_mask, L)) {
       P->words[p] = L.words;
       LaneLayout LL;
-      if (g->lanes && lane_row_ok(row, g->dg.zero_types) && make_lane_layout(L, LL) && lane_pays(L)) {
+      if (g->lanes && lane_row_ok(row, g->dg.zero_types) && make_lane_layout(L, true, LL) && lane_pays(L)) {
         P->lwords[p] = LL.words;
+        make_lane_layout(L, false, LL);
+        P->ltight[p] = LL.words;
         P->lcost[p] = lane_cost(g->dg.work, row, (float)L.NS, (float)(g->node_off[gi + 1] - g->node_off[gi]));
       }
       // per issue the work grows slowly with the simulated SMs; the extended model costs about 3.5x
@@ -2856,27 +2885,26 @@ struct Plan {
   bool sched;  // launch the extended instance (issue policies, NoC, L2)
   bool noc;    // ... with the NoC of DSMEM nodes
   bool lanes;  // lane-parallel instance (every valid row can run there)
+  bool pad;    // ... with padded slots
   float top;   // cost of the dearest row, 0 when every point starts at once
 };
 
 gts_status plan_launch(const gts_graph *g, const gts_params *P, uint32_t first, uint32_t np, uint32_t flags,
                        size_t scratch_bytes, bool limit_by_scratch, Plan &pl) {
   (void)flags;
-  uint32_t words = 64, lwords = 64;
+  uint32_t words = 64, lwords = 64, ltight = 64;
   pl.top = 0.0f;
   pl.sched = false;
   pl.lanes = true;
   for (uint32_t p = first; p < first + np; p++) {
     words = std::max(words, P->words[p]);
     lwords = std::max(lwords, P->lwords[p]);
+    ltight = std::max(ltight, P->ltight[p]);
     pl.top = std::max(pl.top, P->lcost[p]);
     pl.lanes = pl.lanes && (P->lwords[p] || !P->words[p]);
     pl.sched = pl.sched || P->sched[p];
   }
   pl.noc = (g->dg.class_mask & CM_NOC) != 0u;
-  if (pl.lanes) words = lwords;
-  const uint32_t bytes = words * 4;
-  pl.words = words;
   const void *kern = pl.lanes ? (const void *)k_simulate_lanes : pl.noc ? (const void *)k_simulate<true, true>
                    : pl.sched ? (const void *)k_simulate<true, false> : (const void *)k_simulate<false, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM_BYTES);
@@ -2886,18 +2914,37 @@ gts_status plan_launch(const gts_graph *g, const gts_params *P, uint32_t first, 
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return cuda_fail(e, "simulate: kernel attributes");
   // warps per block: whichever keeps the most design points resident per SM
+  auto resident = [&](uint32_t bytes, uint32_t &best_w, uint32_t &best_wpb) {
+    best_w = 0;
+    best_wpb = 1;
+    for (uint32_t wpb = MAX_WPB; wpb >= 1 && e == cudaSuccess; wpb--) {
+      if (wpb * bytes > MAX_SMEM_BYTES) continue;
+      int nb = 0;
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, (int)wpb * 32, wpb * bytes);
+      if ((uint32_t)nb * wpb > best_w) {
+        best_w = (uint32_t)nb * wpb;
+        best_wpb = wpb;
+      }
+    }
+  };
   uint32_t best_w = 0;
-  pl.wpb = 1;
-  for (uint32_t wpb = MAX_WPB; wpb >= 1; wpb--) {
-    if (wpb * bytes > MAX_SMEM_BYTES) continue;
-    int nb = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, (int)wpb * 32, wpb * bytes);
-    if (e != cudaSuccess) return cuda_fail(e, "simulate: occupancy query");
-    if ((uint32_t)nb * wpb > best_w) {
-      best_w = (uint32_t)nb * wpb;
-      pl.wpb = wpb;
+  pl.words = pl.lanes ? lwords : words;
+  pl.pad = true;
+  resident(pl.words * 4, best_w, pl.wpb);
+  if (pl.lanes && ltight < lwords && 2ull * best_w * sms <= np) {
+    // two waves or more: denser slots, where they let more points in (ws GEMM of 3 slots per SM, 9 warps per SM for 7:
+    // 3,000 rows 58.9 ms for 66.3; 1,500 rows, 1.4 waves, 5.10 for 5.01)
+    uint32_t w2 = 0, wpb2 = 1;
+    resident(ltight * 4, w2, wpb2);
+    if (w2 > best_w) {
+      best_w = w2;
+      pl.wpb = wpb2;
+      pl.words = ltight;
+      pl.pad = false;
     }
   }
+  if (e != cudaSuccess) return cuda_fail(e, "simulate: occupancy query");
+  const uint32_t bytes = pl.words * 4;
   uint64_t warps = (uint64_t)std::max(best_w, 1u) * sms;
   // a batch smaller than one wave: one design point per block, so that the
   // block scheduler (which fills SMs breadth first) spreads the points evenly
@@ -2962,7 +3009,7 @@ gts_status gts_simulate_batch(gts_graph *g, gts_params *P, uint32_t first_point,
       k_simulate_lanes<<<pl.blocks, pl.wpb * 32, pl.smem, s>>>(g->dg, P->d_params, first_point, n_points, flags, d_start,
                                                                d_finish, d_makespan, d_status, dig, csm, busy,
                                                                (uint2 *)d_scratch, pl.warps, pl.words, P->d_order, n_order,
-                                                               pl.top);
+                                                               pl.top, pl.pad);
     else
       kern<<<pl.blocks, pl.wpb * 32, pl.smem, s>>>(g->dg, P->d_params, first_point, n_points, flags, d_start, d_finish,
                                                    d_makespan, d_status, dig, csm, busy, (uint2 *)d_scratch, pl.warps,

@@ -147,3 +147,24 @@ def test_points_taken_by_cost_class():
     assert int(full.status.abs().sum()) == 0 and int(part.status.abs().sum()) == 0
     assert torch.equal(full.digest[11:101], part.digest) and torch.equal(full.makespan[11:101], part.makespan)
     assert int(torch.count_nonzero(few[gts.GTS_SCRATCH_HEADER_BYTES:])) == 0
+
+
+@pytest.mark.parametrize("k", [64, 192])
+def test_dense_slots_agree_with_padded_ones(k):
+    """A batch of two waves runs with unpadded slots (3 per SM); its rows in batches of one wave do not."""
+    import torch
+
+    from paper_2607_11262_gb300 import gts
+    g = W.ws_gemm(1024, 1024, k, 132, "ws")
+    p = W.sweep_params(77, 3000, [W.AX_SMS, W.AX_HBM, W.AX_TMA_LAT, W.AX_MMA_RATE], 1)
+    p[0, W.P_NUM_SMS] = 132
+    dg = gts.DeviceGraph(g)
+    dp = gts.DeviceParams(dg, p)
+    flags = gts.GTS_WANT_DIGEST | gts.GTS_WANT_BUSY
+    whole = gts.simulate(dg, dp, flags=flags)
+    for lo in range(0, 3000, 600):
+        part = gts.simulate(dg, dp, first_point=lo, n_points=600, flags=flags)
+        torch.cuda.synchronize()
+        for f in ("status", "makespan", "digest", "busy"):
+            assert torch.equal(getattr(whole, f)[lo:lo + 600], getattr(part, f)), (f, lo)
+    assert int(whole.status.abs().sum()) == 0
