@@ -1315,16 +1315,21 @@ constexpr uint32_t TAG_ID = 0x7FFFFFE0u;
 // meta: pending predecessors << 16 | successors (7: look up) << 13 | type << 10 | byte offset of the SM's servers
 constexpr uint32_t EXHAUSTED = 0xFFFF0000u;
 constexpr uint32_t LANE_DEG_BIG = 7;
+// L2 list in shared memory: head, tail, bytes in use; per tile 16-bit links to the more and the less recent tile
+// (L2_NIL: none; the pair L2_OUT: not listed) and its bytes
+constexpr uint32_t L2_NIL = 0xFFFFu, L2_OUT = 0xFFFEFFFEu, L2_MAX_TILES = 0xFFFDu;
 
 struct LaneLayout {
-  uint32_t Scta, NS, SC, per, per4, cap_hbm;
-  uint32_t o_type, o_slot, o_scout, o_sm, o_list, o_cand, o_cta, o_sv, o_hs, words;
+  uint32_t Scta, NS, SC, per, per4, cap_hbm, nsub;
+  uint32_t o_sub, o_cid, o_type, o_slot, o_scout, o_sm, o_list, o_cand, o_cta, o_l2, o_sv, o_hs, words;
 };
 
 // With `pad`, an SM's slots fill up to a multiple of four with exhausted streams
 // and are read as they lie; without, the last group of four repeats a slot.
-__host__ __device__ inline bool make_lane_layout(const Layout &B, bool pad, LaneLayout &L) {
-  if (B.nsub || B.cap_noc || B.NS > LANE_MAX_SMS || B.per > LANE_MAX_SLOTS) return false;
+// `tiles`: entries of the row's L2 list, 0 without the L2 model.
+__host__ __device__ inline bool make_lane_layout(const Layout &B, bool pad, uint32_t tiles, LaneLayout &L) {
+  if (tiles > L2_MAX_TILES || B.cap_noc || B.NS > LANE_MAX_SMS || B.per > LANE_MAX_SLOTS) return false;
+  L.nsub = B.nsub;
   L.Scta = B.Scta; L.NS = B.NS; L.SC = B.SC + 1; L.per = B.per; L.per4 = pad ? (B.per + 3u) & ~3u : B.per; L.cap_hbm = B.cap_hbm;
   uint64_t w = O_DYN;
   L.o_type = (uint32_t)w; w += 32;
@@ -1332,10 +1337,13 @@ __host__ __device__ inline bool make_lane_layout(const Layout &B, bool pad, Lane
   L.o_scout = (uint32_t)w; w += (uint64_t)L.NS * L.per4;
   w = (w + 3) & ~(uint64_t)3;  // SM records are read as 16-byte vectors
   L.o_sm = (uint32_t)w; w += (uint64_t)L.NS * LANE_SM_WORDS;
-  L.o_list = (uint32_t)w; w += 64 + LANE_CHUNKS;
+  L.o_list = (uint32_t)w; w += 96 + LANE_CHUNKS;
   L.o_cand = (uint32_t)w; w += L.NS;
   w = (w + 1) & ~(uint64_t)1;  // CTA records are read as 8-byte pairs
   L.o_cta = (uint32_t)w; w += (uint64_t)L.Scta * 2;
+  L.o_l2 = (uint32_t)w; w += tiles ? 4ull + 2ull * tiles : 0ull;
+  L.o_sub = (uint32_t)w; w += L.nsub ? (uint64_t)L.NS * (L.nsub + 1u) * SUB_WORDS : 0u;  // and the SM's last issue
+  L.o_cid = (uint32_t)w; w += L.nsub ? L.Scta : 0u;
   L.o_sv = (uint32_t)w; w += (uint64_t)L.NS * L.SC;
   L.o_hs = (uint32_t)w; w += L.cap_hbm;
   w = (w + 3) & ~(uint64_t)3;
@@ -1347,11 +1355,11 @@ __host__ __device__ inline bool make_lane_layout(const Layout &B, bool pad, Lane
 // A row whose nodes all take at least one cycle: zero_types has a bit per type
 // with a node of no work (or a NOP) and no extra latency.
 __host__ __device__ inline bool lane_row_ok(const int32_t *p, uint32_t zero_types) {
-  const int64_t base[8] = {(int64_t)p[GTS_P_TMA_LAT] + p[GTS_P_DRAM_LAT], p[GTS_P_SMEM_LAT], p[GTS_P_MMA_LAT],
-                           p[GTS_P_ALU_LAT], p[GTS_P_TMA_LAT], 1, 0, 0};
+  const int64_t load = (int64_t)p[GTS_P_TMA_LAT] + (p[GTS_P_L2_BYTES] ? p[GTS_P_L2_LAT] : p[GTS_P_DRAM_LAT]);
+  const int64_t base[8] = {load, p[GTS_P_SMEM_LAT], p[GTS_P_MMA_LAT], p[GTS_P_ALU_LAT], p[GTS_P_TMA_LAT], 1, 0, 0};
   for (int k = 0; k < 8; k++)
     if (((zero_types >> k) & 1u) && base[k] == 0) return false;
-  return p[GTS_P_ISSUE_POLICY] == GTS_POLICY_LOWEST_ID && p[GTS_P_L2_BYTES] == 0;
+  return true;
 }
 
 // Rows of one SM leave the lanes nothing to share: the one-SM pipeline study (1,536
@@ -1422,6 +1430,10 @@ struct LanePt {
   uint64_t offs;  // byte k: offset, on an SM, of the servers of type k (the last word, always 0, for NOP)
   uint32_t caps;  // 6 bits per class
   uint32_t off_ld, cap_tma;  // servers of LOAD and STORE
+  uint32_t policy, mSub;
+  __device__ __forceinline__ uint32_t *sub(uint32_t s, uint32_t u) const {
+    return sp + L.o_sub + (s * (L.nsub + 1u) + u) * SUB_WORDS;
+  }
   uint32_t mW, mCps;
   __device__ __forceinline__ uint4 *slots(uint32_t s) const {
     return reinterpret_cast<uint4 *>(sp + L.o_slot + s * (L.per4 * LANE_SLOT_WORDS));
@@ -1529,6 +1541,79 @@ __device__ __forceinline__ void lane_refresh(const LanePt &P, uint32_t s, uint32
   P.smrec(s)[1] = b;
 }
 
+// As lane_refresh, under the per-subpartition schedulers (Section 5.3).  Scheduler
+// u's event is E_u = max(first cycle it may issue, least key of its heads, a waiting
+// head's being max(key, H)); its pick is the first head in policy order with a key
+// up to E_u.  A pick that waits for no HBM server stays the pick whatever becomes of
+// H, one that does is lost when H passes E_u.  So the record holds the SM's first
+// event (E_u, id) alone: as its first head when no waiting pick comes in the same
+// cycle, else as a candidate for the global order -- the waiting pick itself, or the
+// lower id that issues before it -- out of date once H passes its cycle, unless it is
+// the SM's only head that could issue.
+// A pick may show up late in its cycle, when a node of higher id has taken a unit of
+// the pick before it: its place in the global order is after that node.  b.w is the
+// tag of that place; of a first head, as long as H has not passed its cycle, a bound
+// on the places of the HBM heads to come.
+__device__ __forceinline__ void lane_refresh_sub(const LanePt &P, uint32_t s, uint32_t H, uint4 &a, uint4 &b) {
+  const uint32_t *sv = P.servers(s);
+  const uint4 *sl = P.slots(s);
+  uint64_t first = INF64;
+  uint32_t wait_e = INF, heads = 0;
+  bool waits = false;
+  auto key = [&](const uint4 &q) {  // INF: cannot issue
+    if (q.y >= (1u << 16)) return INF;
+    const uint32_t k = max(q.x, *reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(sv) + (q.y & 1023u)));
+    return (int32_t)q.z < 0 ? max(k, H) : k;
+  };
+#pragma unroll 1
+  for (uint32_t u = 0; u < P.L.nsub; u++) {
+    uint32_t m = INF;
+#pragma unroll 2
+    for (uint32_t l = u; l < P.L.per; l += P.L.nsub) {
+      const uint32_t k = key(sl[2 * l]);
+      m = min(m, k);
+      heads += k != INF ? 1u : 0u;
+    }
+    if (m == INF) continue;
+    const uint32_t *sq = P.sub(s, u);
+    const uint32_t E = max(m, sq[Q_AVAIL]), last = sq[Q_LAST];
+    uint32_t best = INF, tag = 0;
+#pragma unroll 2
+    for (uint32_t l = u; l < P.L.per; l += P.L.nsub) {
+      const uint4 q = sl[2 * l];
+      if (key(q) > E) continue;
+      uint32_t order;
+      if (P.policy == GTS_POLICY_GTO) {  // greedy slot, then the oldest warp (CTA id, warp)
+        const uint32_t jl = P.cps > 1u ? div16(l, P.mW) : 0u;
+        order = (l == last ? 0u : 0x80000000u) | (P.sp[P.L.o_cid + s * P.cps + jl] * P.W + (l - jl * P.W));
+      } else {  // round-robin after the last slot
+        const uint32_t x = l + P.L.per - last - 1u;
+        order = last == NONE ? l : (x >= P.L.per ? x - P.L.per : x);
+      }
+      if (order <= best) {
+        best = order;
+        tag = q.z;
+      }
+    }
+    const bool w = (int32_t)tag < 0;
+    if (w) wait_e = min(wait_e, E);
+    const uint64_t e = pack(E, tag & ID_MASK);
+    if (e < first) {
+      first = e;
+      waits = w;
+    }
+  }
+  const uint32_t E = (uint32_t)(first >> 32), tag = (uint32_t)first;
+  const bool cand = waits || (first != INF64 && wait_e == E);
+  a = cand ? make_uint4(INF, NONE, E, tag) : make_uint4(E, tag, INF, NONE);
+  b.y = cand ? INF : max(E, sv[P.off_ld]);
+  b.z = cand && heads > 1u ? E + 1u : INF;
+  const uint32_t *done = P.sub(s, P.L.nsub);  // cycle of the SM's last issue, highest tag that issued in it
+  b.w = E == done[0] ? max(tag, done[1]) : tag;
+  P.smrec(s)[0] = a;
+  P.smrec(s)[1] = b;
+}
+
 // The part of SM s's record that changes with its CTAs.
 __device__ __forceinline__ void lane_ctas(const LanePt &P, uint32_t s, uint4 &b) {
   uint32_t U = INF;
@@ -1541,9 +1626,10 @@ __device__ __forceinline__ void lane_ctas(const LanePt &P, uint32_t s, uint4 &b)
 }
 
 // Whether SM record (a, b)'s first head may issue: before its SM's waiting HBM
-// head and not past a retirement that will launch a CTA (U).
+// head and not past a retirement that will launch a CTA (U; under the schedulers of
+// a policy before it, as the new CTA's heads may change their picks).
 __device__ __forceinline__ bool lane_issuable(const uint4 &a, uint32_t H, uint32_t U) {
-  return a.x <= U && pack(a.x, a.y) < pack(max(a.z, H), a.w);
+  return a.x <= U && pack(a.x, a.y) < pack(max(a.z, H), a.w);  // false without a first head (no cycle is INF)
 }
 
 // ceil(n / d) given M = div_const(d), as cdiv_c, without branches.
@@ -1641,6 +1727,7 @@ __device__ __forceinline__ void lane_launch(const DevGraph &g, const LanePt &P, 
       const uint32_t s = div16(j, P.mCps);
       *P.cta(j) = make_uint2(cnt, 0u);
       P.smrec(s)[1].z = 0u;
+      if (P.L.nsub) P.sp[P.L.o_cid + j] = c;
       list[rank] = j;
       if (cta_sm_row) cta_sm_row[c - P.c0] = (int32_t)s;
     }
@@ -1669,10 +1756,11 @@ __device__ __forceinline__ void lane_launch(const DevGraph &g, const LanePt &P, 
 }
 
 // Issues SM s's first head (record a) at its key; the record is then out of date.
-// Returns the finish cycle, 2^31 or more on overflow (nothing is changed then).
+// hit_lat: latency of a LOAD that hit in L2, else NONE.  Returns the finish cycle,
+// 2^31 or more on overflow (nothing is changed then).
 // The loads are started first; the server, CTA and trace updates need none of them.
 __device__ __forceinline__ uint32_t lane_issue(const DevGraph &g, const LanePt &P, uint32_t s, uint64_t pol,
-                                               const uint4 &a, bool &cta_done) {
+                                               const uint4 &a, uint32_t hit_lat, bool &cta_done) {
   const uint32_t t = a.x, l = a.y & 31u, v = a.y >> 5;
   uint4 *sl = P.slots(s);
   const uint4 q = sl[2 * l], z = sl[2 * l + 1];
@@ -1696,7 +1784,7 @@ __device__ __forceinline__ uint32_t lane_issue(const DevGraph &g, const LanePt &
     cn = ld_counters_keep(counters, pol);
     if (scan) sr = ld_next_type(g.rec, at);
   }
-  const uint32_t f = t + z.w, off = (q.y & 1023u) >> 2;
+  const uint32_t f = t + (hit_lat != NONE ? hit_lat : z.w), off = (q.y & 1023u) >> 2;
   if ((int32_t)f < 0) return f;
   if (off != P.L.SC - 1u) take_server(P.servers(s) + off, (q.y & (3u << 10)) ? z.y : P.cap_tma, t + z.x);
   if (P.st) {
@@ -1750,6 +1838,45 @@ __device__ __forceinline__ uint32_t lane_issue(const DevGraph &g, const LanePt &
   return f;
 }
 
+// One access of a point's L2 list (Section 5.2), as l2_access, on the list in
+// shared memory: tile x becomes the most recent entry, sized b.  Whether it was
+// listed (a hit).  One lane calls it.
+__device__ __forceinline__ bool lane_l2_access(uint32_t *st, uint32_t x, uint32_t b, uint64_t cap) {
+  uint32_t *T = st + 4;
+  auto link = [&](uint32_t k) { return reinterpret_cast<uint16_t *>(T + 2u * k); };  // [0] more recent, [1] less recent
+  uint32_t head = st[0], tail = st[1];
+  uint64_t used = *reinterpret_cast<const uint64_t *>(st + 2);
+  const uint2 e = *reinterpret_cast<const uint2 *>(T + 2u * x);
+  const bool hit = e.x != L2_OUT;
+  if (hit) {
+    const uint32_t more = e.x & 0xFFFFu, less = e.x >> 16;
+    if (more != L2_NIL) link(more)[1] = (uint16_t)less; else head = less;
+    if (less != L2_NIL) link(less)[0] = (uint16_t)more; else tail = more;
+    used -= e.y;
+  }
+  *reinterpret_cast<uint2 *>(T + 2u * x) = make_uint2(L2_NIL | head << 16, b);
+  if (head != L2_NIL) link(head)[0] = (uint16_t)x; else tail = x;
+  head = x;
+  used += b;
+#pragma unroll 1
+  while (used > cap) {  // every entry dropped leaves used <= cap at the latest
+    const uint2 d = *reinterpret_cast<const uint2 *>(T + 2u * tail);
+    T[2u * tail] = L2_OUT;
+    tail = d.x & 0xFFFFu;
+    if (tail != L2_NIL) link(tail)[1] = (uint16_t)L2_NIL; else head = L2_NIL;
+    used -= d.y;
+  }
+  st[0] = head;
+  st[1] = tail;
+  *reinterpret_cast<uint64_t *>(st + 2) = used;
+  return hit;
+}
+
+struct LaneL2 {  // per lane: HBM server-cycles, LOAD hits, LOADs that named a tile
+  uint64_t hbm, cap;  // cap: the row's L2 bytes, 0 without the model
+  uint32_t hits, loads;
+};
+
 // HBM grants in (cycle, id) order while the first candidate precedes every bound;
 // then the task list: the granted SMs with their cycles, and those whose first head
 // H passed.  Per lane CH SMs with a waiting head in registers, each with two
@@ -1759,18 +1886,23 @@ __device__ __forceinline__ uint32_t lane_issue(const DevGraph &g, const LanePt &
 // the SM waits for a TMA server.  It may precede earlier heads of its SM that use
 // other units: their issue does not depend on it, and it not on theirs.  Returns
 // the SMs granted (at most 32, one task each), NONE on overflow.
-template <uint32_t CH>
-__device__ __forceinline__ uint32_t lane_grant(const LanePt &P, uint32_t &H, bool live, int lane, uint32_t n_cand,
+// With the L2 model a grant is also the access of its node's tile: a hit takes
+// the server for ceil(work / l2_bpc) cycles, and its latency goes with the task.
+template <uint32_t CH, bool EXT>
+__device__ __forceinline__ uint32_t lane_grant(const DevGraph &g, const LanePt &P, LaneL2 &X, uint32_t &H, bool live,
+                                               int lane, uint32_t n_cand,
                                                uint32_t min_u, uint32_t lb_h, uint32_t lb_i, uint32_t lb_2,
                                                uint32_t lb_any, uint32_t &n_task) {
   const uint32_t below = (1u << lane) - 1u;
   uint32_t K[CH], ID[CH], L[CH], IM[CH], K2[CH], HO[CH], OC[CH];
-  uint32_t granted = 0, n_granted = 0;
+  uint32_t TI[CH], BY[CH], HH[CH], LH[CH];  // L2 model: tile + 1 << 1 | LOAD, bytes, HBM cycles and latency of a hit
+  uint32_t granted = 0, n_granted = 0, no_server = 0;
 #pragma unroll
   for (uint32_t c = 0; c < CH; c++) {
     K[c] = L[c] = K2[c] = INF;
     ID[c] = IM[c] = NONE << 1;
     HO[c] = OC[c] = 0;
+    if (EXT) TI[c] = BY[c] = HH[c] = 0, LH[c] = NONE;
     if (32u * c + lane < n_cand) {
       const uint32_t s = P.sp[P.L.o_cand + 32u * c + lane];
       const uint4 a = P.smrec(s)[0], b = P.smrec(s)[1];
@@ -1784,15 +1916,35 @@ __device__ __forceinline__ uint32_t lane_grant(const LanePt &P, uint32_t &H, boo
       K2[c] = b.z;
       HO[c] = o.y;
       OC[c] = P.cap_tma == 1u ? o.x : 0u;
+      if (EXT && P.L.nsub) {
+        // a head that waits for no server takes part for the order alone; SMs with a pending launch wait for it
+        const bool w = (int32_t)P.slots(s)[2 * (a.w & 31u)].z < 0;
+        ID[c] = b.w << 1 | (max(a.z, H) < U || U == INF ? 1u : 0u);
+        if (!w) {
+          no_server |= 1u << c;
+          OC[c] = 0u;
+        }
+      }
+      if (EXT && X.cap) {
+        const uint32_t v = P.n0 + (a.w >> 5);
+        const uint2 wl = *reinterpret_cast<const uint2 *>(g.rec + v);
+        const bool load = ((P.slots(s)[2 * (a.w & 31u)].y >> 10) & 7u) == GTS_LOAD;
+        TI[c] = g.rng[v].x << 1 | (load ? 1u : 0u);
+        BY[c] = wl.x;
+        HH[c] = cdiv_flat(wl.x, P.sp[GTS_P_L2_BPC], P.sp[O_MAG + 12], P.sp[O_MAG + 13]);
+        const uint64_t lat = (uint64_t)P.sp[O_L2B] + wl.y + max(o.x, HH[c]);
+        LH[c] = lat > 0x80000000ull ? 0x80000000u : (uint32_t)lat;
+      }
     }
   }
 #pragma unroll 1
   while (n_granted < 32u) {
     const uint32_t ux = max(min_u, H);
     uint32_t x = max(lb_h, H), y = H > lb_h && H >= lb_2 ? lb_any : lb_i, at = 0;
-    if (pack(ux, 0xFFFFFFFEu) < pack(x, y)) {
+    const uint32_t uy = EXT && P.L.nsub ? 0u : 0xFFFFFFFEu;  // a launch may change a scheduler's pick
+    if (pack(ux, uy) < pack(x, y)) {
       x = ux;
-      y = 0xFFFFFFFEu;
+      y = uy;
     }
 #pragma unroll
     for (uint32_t c = 0; c < CH; c++) {
@@ -1816,8 +1968,29 @@ __device__ __forceinline__ uint32_t lane_grant(const LanePt &P, uint32_t &H, boo
     uint32_t ho = HO[0];
 #pragma unroll
     for (uint32_t c = 1; c < CH; c++) ho = at == c ? HO[c] : ho;
+    bool missed = true;
+    if (EXT && win && ((no_server >> at) & 1u)) {
+      ho = NONE;
+    } else if (EXT && X.cap) {
+      if (win) {
+        uint32_t ti = TI[0], by = BY[0], hh = HH[0];
+#pragma unroll
+        for (uint32_t c = 1; c < CH; c++) {
+          ti = at == c ? TI[c] : ti;
+          by = at == c ? BY[c] : by;
+          hh = at == c ? HH[c] : hh;
+        }
+        const bool tile = ti > 1u, hit = tile && lane_l2_access(P.sp + P.L.o_l2, (ti >> 1) - 1u, by, X.cap);
+        missed = !(hit && (ti & 1u));
+        ho = missed ? ho : hh;
+        X.hbm += ho;
+        X.hits += missed ? 0u : 1u;
+        X.loads += tile ? ti & 1u : 0u;
+      }
+    }
     ho = __reduce_max_sync(FULL, win ? ho : 0u);
-    if ((uint64_t)t + ho > 0x7FFFFFFFull) return NONE;
+    const bool takes = !EXT || ho != NONE;
+    if (takes && (uint64_t)t + ho > 0x7FFFFFFFull) return NONE;
     n_granted++;
     granted |= win ? 1u << at : 0u;
 #pragma unroll
@@ -1828,7 +2001,9 @@ __device__ __forceinline__ uint32_t lane_grant(const LanePt &P, uint32_t &H, boo
       K[c] = mine ? INF : K[c];
       K2[c] = mine ? INF : K2[c];
       HO[c] = mine ? t : HO[c];
+      if (EXT) LH[c] = mine && missed ? NONE : LH[c];
     }
+    if (!takes) continue;
     if (P.L.cap_hbm == 1u) {
       H = t + ho;
     } else {
@@ -1840,7 +2015,7 @@ __device__ __forceinline__ uint32_t lane_grant(const LanePt &P, uint32_t &H, boo
       H = __reduce_min_sync(FULL, hv);
     }
   }
-  uint32_t *listed = P.sp + P.L.o_list + 64;
+  uint32_t *listed = P.sp + P.L.o_list + 96;
 #pragma unroll
   for (uint32_t c = 0; c < CH; c++) {
     if (32u * c < n_cand) {
@@ -1851,6 +2026,7 @@ __device__ __forceinline__ uint32_t lane_grant(const LanePt &P, uint32_t &H, boo
         uint32_t *li = P.sp + P.L.o_list + n_task + __popc(bal & below);
         li[0] = s;
         li[32] = HO[c];
+        if (EXT) li[64] = X.cap ? LH[c] : NONE;
         atomicOr(listed + (s >> 5), 1u << (s & 31u));
       }
       n_task += __popc(bal);
@@ -1872,6 +2048,10 @@ __device__ __forceinline__ uint32_t lane_grant(const LanePt &P, uint32_t &H, boo
   return n_granted;
 }
 
+// EXT: the instance for tables with rows under the L2 model or an issue policy
+// (96 rows of the L2 study's GEMM 8.97 ms, 66.1 in k_simulate<true, false>; 448 rows
+// of the policy study 12.2 for 17.2).
+template <bool EXT>
 __global__ void __launch_bounds__(MAX_WPB * 32, 3)
 k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__ params, uint32_t first_point, uint32_t n_points, uint32_t flags,
                  int32_t *d_start, int32_t *d_finish, int32_t *d_makespan, int32_t *d_status, uint64_t *d_digest,
@@ -1908,7 +2088,8 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
     const uint32_t CG = P.c1 - P.c0;
     if (status == GTS_OK) {
       Layout B;
-      if (!make_layout(prm, CG, P.W, g.class_mask, B) || !make_lane_layout(B, pad, P.L) || P.L.words > budget_words ||
+      if (!make_layout(prm, CG, P.W, g.class_mask, B) || (!EXT && (prm[GTS_P_L2_BYTES] || B.nsub)) ||
+          !make_lane_layout(B, pad, prm[GTS_P_L2_BYTES] ? g.n_tiles : 0u, P.L) || P.L.words > budget_words ||
           !lane_row_ok(prm, g.zero_types))
         status = GTS_ERR_UNSUPPORTED;
     }
@@ -1953,7 +2134,9 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
       const uint32_t rt = (TYPE_RATE >> (4 * lane)) & 15u;
       const uint64_t M = rt < 5u ? *reinterpret_cast<const uint64_t *>(sp + O_MAG + 2 * rt) : 0ull;
       *reinterpret_cast<uint4 *>(sp + P.L.o_type + 4 * lane) =
-          make_uint4(rt < 5u ? sp[GTS_P_HBM_BPC + 2 * rt] : 1u, sp[O_BASE + lane], (uint32_t)M, (uint32_t)(M >> 32));
+          make_uint4(rt < 5u ? sp[GTS_P_HBM_BPC + 2 * rt] : 1u,
+                     EXT && lane == GTS_LOAD && prm[GTS_P_L2_BYTES] ? sp[O_L2B + 1] : sp[O_BASE + lane], (uint32_t)M,
+                     (uint32_t)(M >> 32));
     }
     for (uint32_t i = lane; i < P.L.NS * P.L.per4; i += 32) {
       P.slots(0)[2 * i] = make_uint4(0u, EXHAUSTED, ID_MASK, NONE);
@@ -1978,6 +2161,27 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
     __threadfence();
     __syncwarp();
 
+    P.policy = (uint32_t)prm[GTS_P_ISSUE_POLICY];
+    P.mSub = div16_const(P.L.nsub);
+    const uint32_t before = EXT && P.L.nsub ? 1u : 0u;
+    if (EXT)
+      for (uint32_t k = lane; k < (P.L.nsub ? P.L.NS * (P.L.nsub + 1u) : 0u); k += 32) {
+        sp[P.L.o_sub + k * SUB_WORDS + Q_AVAIL] = 0u;
+        sp[P.L.o_sub + k * SUB_WORDS + Q_LAST] = (k + 1u) % (P.L.nsub + 1u) ? NONE : 0u;
+      }
+    LaneL2 X;
+    X.hbm = X.cap = 0;
+    X.hits = X.loads = 0;
+    if (EXT && prm[GTS_P_L2_BYTES]) {
+      X.cap = (uint64_t)prm[GTS_P_L2_BYTES];
+      uint32_t *st = sp + P.L.o_l2;
+      for (uint32_t k = lane; k < g.n_tiles; k += 32) st[4 + 2 * k] = L2_OUT;
+      if (lane == 0 && g.n_tiles) {
+        st[0] = st[1] = L2_NIL;
+        *reinterpret_cast<uint64_t *>(st + 2) = 0ull;
+      }
+      __syncwarp();
+    }
     LaneState Q;
     Q.next = P.c0;
     Q.nres = Q.nrun = Q.kernel = 0;
@@ -2017,12 +2221,13 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
           b = P.smrec(s)[1];
         }
         const uint32_t U = live ? b.x : INF, e = max(a.z, H);
-        const bool iss = lane_issuable(a, H, U);
+        const bool iss = lane_issuable(a, H, U - before);
         mask |= (iss ? 1u : 0u) << c;
         min_u = min(min_u, U);
         min_e = min(min_e, min(a.x, e));
         const bool cand = a.z != INF, bounds = !cand && a.x != INF;
-        const uint32_t x = bounds ? max(b.y, H) : INF, y = bounds ? b.w : NONE;
+        uint32_t x = bounds ? max(b.y, H) : INF, y = bounds ? b.w : NONE;
+        if (EXT && P.L.nsub && x != a.x) y = x != INF ? 0u : NONE;
         const bool less = pack(x, y) < pack(lb_h, lb_i);
         lb_2 = min(lb_2, less ? lb_h : x);
         lb_h = less ? x : lb_h;
@@ -2039,7 +2244,7 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
           n_task += __popc(sb);
         }
       }
-      if (lane < (int)LANE_CHUNKS) sp[P.L.o_list + 64 + lane] = 0u;  // SMs already in the task list
+      if (lane < (int)LANE_CHUNKS) sp[P.L.o_list + 96 + lane] = 0u;  // SMs already in the task list
       __syncwarp();
       const bool refresh_only = n_task != 0u;
       uint32_t n_granted = 0;
@@ -2062,15 +2267,16 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
         }
         lb_i <<= 1;
         lb_any <<= 1;
+        if (EXT && P.L.nsub) lb_2 = lb_any = 0u;
         // (two candidates per lane apart: 65.2 for 67.2 ms on the wide ws GEMM table)
-        n_granted = n_cand <= 32u   ? lane_grant<1>(P, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task)
-                    : n_cand <= 64u ? lane_grant<2>(P, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task)
-                                    : lane_grant<LANE_CHUNKS>(P, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task);
+        n_granted = n_cand <= 32u   ? lane_grant<1, EXT>(g, P, X, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task)
+                    : n_cand <= 64u ? lane_grant<2, EXT>(g, P, X, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task)
+                                    : lane_grant<LANE_CHUNKS, EXT>(g, P, X, H, live, lane, n_cand, min_u, lb_h, lb_i, lb_2, lb_any, n_task);
         if (n_granted == NONE) { status = GTS_ERR_OVERFLOW; break; }
         __syncwarp();
 #pragma unroll 1
         for (uint32_t s = lane, c = 0; s - lane < P.L.NS && n_task < 32u; s += 32, c++) {
-          const bool go = ((mask >> c) & 1u) && !((sp[P.L.o_list + 64 + c] >> lane) & 1u);
+          const bool go = ((mask >> c) & 1u) && !((sp[P.L.o_list + 96 + c] >> lane) & 1u);
           const uint32_t bal = __ballot_sync(FULL, go), at = n_task + __popc(bal & below);
           if (go && at < 32u) sp[P.L.o_list + at] = s;
           n_task += __popc(bal);
@@ -2083,6 +2289,7 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
       bool act = (uint32_t)lane < n_task;
       uint32_t s = 0;
       uint4 a = make_uint4(INF, NONE, INF, NONE), b = a;
+      uint32_t hit_lat = NONE;
       if (act) {
         s = sp[P.L.o_list + lane];
         a = P.smrec(s)[0];
@@ -2090,8 +2297,9 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
         if ((uint32_t)lane < n_granted) {  // its waiting head issues at the cycle of its grant
           a.x = sp[P.L.o_list + 32 + lane];
           a.y = a.w;
+          if (EXT) hit_lat = sp[P.L.o_list + 64 + lane];
         } else {
-          act = refresh_only || lane_issuable(a, H, live ? b.x : INF);
+          act = refresh_only || lane_issuable(a, H, (live ? b.x : INF) - before);
         }
       }
       n_task = __popc(__ballot_sync(FULL, act));
@@ -2102,20 +2310,31 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
         bool done = false;
         if (act) {
           if (!refresh_only) {
-            const uint32_t f = lane_issue(g, P, s, pol, a, done);
+            const uint32_t f = lane_issue(g, P, s, pol, a, hit_lat, done);
+            hit_lat = NONE;
+            if (EXT && P.L.nsub) {  // the issuing scheduler: one issue per cycle, remember the slot
+              const uint32_t l = a.y & 31u;
+              uint32_t *sq = P.sub(s, l - div16(l, P.mSub) * P.L.nsub);
+              sq[Q_AVAIL] = a.x + 1u;
+              sq[Q_LAST] = l;
+              uint32_t *last = P.sub(s, P.L.nsub);
+              last[1] = last[0] == a.x ? max(last[1], a.y & ID_MASK) : a.y & ID_MASK;
+              last[0] = a.x;
+            }
             over |= (int32_t)f < 0;
             mk = max(mk, f);
             tlast = max(tlast, a.x);
             if (want_digest) digest += mix64(((uint64_t)(a.y >> 5) << 32 | a.x) ^ ((uint64_t)f * 0x9E3779B97F4A7C15ull));
           }
           if (done || refresh_only) lane_ctas(P, s, b);
-          lane_refresh(P, s, H, a, b);
+          if (EXT && P.L.nsub) lane_refresh_sub(P, s, H, a, b);
+          else lane_refresh(P, s, H, a, b);
         }
         __syncwarp();
         if (refresh_only) break;
         issued += left;
         Q.nrun -= __popc(__ballot_sync(FULL, done));
-        act = act && !over && lane_issuable(a, H, live ? b.x : INF);
+        act = act && !over && lane_issuable(a, H, (live ? b.x : INF) - before);
         left = __popc(__ballot_sync(FULL, act));
         if (left == 0u) break;
       }
@@ -2147,12 +2366,17 @@ k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__
           for (uint32_t k = 0; k < RC_N; k++) busy[k] += cls == k ? occ : 0u;
           busy[5] += hocc;
         }
+        if (EXT && X.cap) busy[5] = X.hbm;
       }
       uint64_t x = 0;
 #pragma unroll
       for (uint32_t k = 0; k < 6; k++) {
         for (int o = 16; o > 0; o >>= 1) busy[k] += __shfl_xor_sync(FULL, busy[k], o);
         x = (uint32_t)lane == k ? busy[k] : x;
+      }
+      if (EXT && status == GTS_OK) {
+        const uint32_t hits = __reduce_add_sync(FULL, X.hits), loads = __reduce_add_sync(FULL, X.loads);
+        x = lane == GTS_BUSY_L2_HITS ? hits : lane == GTS_BUSY_L2_LOADS ? loads : x;
       }
       if (lane < GTS_BUSY_CLASSES) d_busy[(size_t)q * GTS_BUSY_CLASSES + lane] = (int64_t)x;
     }
@@ -2837,9 +3061,10 @@ gts_status gts_params_upload(gts_graph *g, const int32_t *d_params, uint32_t n_p
     if (make_layout(row, g->cta_off[gi + 1] - g->cta_off[gi], g->W, g->dg.class_mask, L)) {
       P->words[p] = L.words;
       LaneLayout LL;
-      if (g->lanes && lane_row_ok(row, g->dg.zero_types) && make_lane_layout(L, true, LL) && lane_pays(L)) {
+      if (g->lanes && lane_row_ok(row, g->dg.zero_types) && make_lane_layout(L, true, row[GTS_P_L2_BYTES] ? g->dg.n_tiles : 0u, LL) &&
+          lane_pays(L)) {
         P->lwords[p] = LL.words;
-        make_lane_layout(L, false, LL);
+        make_lane_layout(L, false, row[GTS_P_L2_BYTES] ? g->dg.n_tiles : 0u, LL);
         P->ltight[p] = LL.words;
         P->lcost[p] = lane_cost(g->dg.work, row, (float)L.NS, (float)(g->node_off[gi + 1] - g->node_off[gi]));
       }
@@ -2905,7 +3130,8 @@ gts_status plan_launch(const gts_graph *g, const gts_params *P, uint32_t first, 
     pl.sched = pl.sched || P->sched[p];
   }
   pl.noc = (g->dg.class_mask & CM_NOC) != 0u;
-  const void *kern = pl.lanes ? (const void *)k_simulate_lanes : pl.noc ? (const void *)k_simulate<true, true>
+  const void *kern = pl.lanes ? (pl.sched ? (const void *)k_simulate_lanes<true> : (const void *)k_simulate_lanes<false>)
+                   : pl.noc ? (const void *)k_simulate<true, true>
                    : pl.sched ? (const void *)k_simulate<true, false> : (const void *)k_simulate<false, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
@@ -3005,15 +3231,16 @@ gts_status gts_simulate_batch(gts_graph *g, gts_params *P, uint32_t first_point,
     int32_t *csm = (flags & GTS_WANT_CTA_SM) ? d_cta_sm : nullptr;
     int64_t *busy = (flags & GTS_WANT_BUSY) ? d_busy : nullptr;
     const uint32_t n_order = P->d_order ? P->n_points : 0u;
-    if (pl.lanes)
-      k_simulate_lanes<<<pl.blocks, pl.wpb * 32, pl.smem, s>>>(g->dg, P->d_params, first_point, n_points, flags, d_start,
-                                                               d_finish, d_makespan, d_status, dig, csm, busy,
-                                                               (uint2 *)d_scratch, pl.warps, pl.words, P->d_order, n_order,
-                                                               pl.top, pl.pad);
-    else
+    if (pl.lanes) {
+      auto lanes = pl.sched ? k_simulate_lanes<true> : k_simulate_lanes<false>;
+      lanes<<<pl.blocks, pl.wpb * 32, pl.smem, s>>>(g->dg, P->d_params, first_point, n_points, flags, d_start, d_finish,
+                                                    d_makespan, d_status, dig, csm, busy, (uint2 *)d_scratch, pl.warps,
+                                                    pl.words, P->d_order, n_order, pl.top, pl.pad);
+    } else {
       kern<<<pl.blocks, pl.wpb * 32, pl.smem, s>>>(g->dg, P->d_params, first_point, n_points, flags, d_start, d_finish,
                                                    d_makespan, d_status, dig, csm, busy, (uint2 *)d_scratch, pl.warps,
                                                    pl.words, P->d_order, n_order);
+    }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "simulate: launch");
   }

@@ -1,10 +1,10 @@
 """The lane-parallel kernel instance (one simulated SM per lane), which the
-library launches when every valid row has the lowest-id order on at least two
-SMs and the graph's ids are in CTA order with no edge between CTAs: against the
-oracle where its tiles end (SMs per lane round, slots read four at a time, the
-inline successors, servers kept in registers up to four), and against the
-general instance, which the same rows run in when the batch also holds a row of
-one SM.  Integer results, compared bit for bit."""
+library launches when every valid row has at least two SMs and the graph's ids
+are in CTA order with no edge between CTAs: against the oracle where its tiles
+end (SMs per lane round, slots read four at a time, the inline successors,
+servers kept in registers up to four, L2 lists in shared memory), and against
+the general instance, which the same rows run in when the batch also holds a row
+of one SM.  Integer results, compared bit for bit."""
 import numpy as np
 import pytest
 
@@ -168,3 +168,60 @@ def test_dense_slots_agree_with_padded_ones(k):
         for f in ("status", "makespan", "digest", "busy"):
             assert torch.equal(getattr(whole, f)[lo:lo + 600], getattr(part, f)), (f, lo)
     assert int(whole.status.abs().sum()) == 0
+
+
+def _with_l2(rng, p, tiles_bytes):
+    p = p.copy()
+    p[W.P_L2_BYTES], p[W.P_L2_LAT], p[W.P_L2_BPC] = int(rng.choice(tiles_bytes)), int(rng.integers(1, 9)), int(rng.choice([1, 2, 5]))
+    return p
+
+
+@pytest.mark.parametrize("tiles", [1, 7, 64, 3000, 65533, 65534])
+def test_l2_lists(tiles):
+    """The L2 list in shared memory, up to its largest tile count (and one more, which the general instance runs)."""
+    rng = np.random.default_rng(7600 + tiles)
+    for mix in (0, 2):
+        g = _graph(rng, 220, 24, 3, mix, kernels=mix == 2)
+        g.tile = rng.integers(max(0, tiles - 40), tiles, g.n_nodes).astype(np.uint32)
+        g.tile[::6] = W.NO_TILE
+        g.n_tiles = tiles
+        rows = [_row(rng, int(rng.choice([2, 5, 40])), int(rng.integers(1, 3)), int(rng.integers(1, 3))) for _ in range(5)]
+        rows = np.stack([rows[0]] + [_with_l2(rng, p, [1, 6, 30, 10**6]) for p in rows[1:]])
+        _check(g, rows, H.run_gpu(g, rows))
+
+
+@pytest.mark.parametrize("schedulers", [1, 2, 3, 4, 7, 32])
+@pytest.mark.parametrize("policy", [W.POLICY_GTO, W.POLICY_RR])
+def test_issue_policies(policy, schedulers):
+    """Schedulers of a policy in the lanes, beside lowest-id rows and rows with an L2 list."""
+    rng = np.random.default_rng(7700 + 40 * policy + schedulers)
+    for mix in range(4):
+        g = _graph(rng, 260, 30, 4, mix, kernels=mix == 1, p_issue=[0.0, 0.3, 0.8, 0.3][mix])
+        g.tile = rng.integers(0, 9, g.n_nodes).astype(np.uint32)
+        g.n_tiles = 9
+        rows = []
+        for k in range(6):
+            p = _row(rng, int(rng.choice([2, 3, 8, 33])), int(rng.choice([1, 2, 4])), int(rng.choice([1, 2])),
+                     int(rng.choice([1, 3])))
+            if k:
+                p[W.P_ISSUE_POLICY], p[W.P_SUBPARTITIONS] = policy, schedulers
+            rows.append(_with_l2(rng, p, [8, 40]) if k == 5 else p)
+        rows = np.stack(rows)
+        _check(g, rows, H.run_gpu(g, rows))
+
+
+@pytest.mark.parametrize("seed", range(4))
+def test_policies_agree_with_the_general_instance(seed):
+    rng = np.random.default_rng(7800 + seed)
+    g = _graph(rng, 500, 50, int(rng.integers(2, 6)), seed, max_work=[2, 6, 60, 6][seed])
+    rows = []
+    for k in range(24):
+        p = _row(rng, int(rng.choice([2, 5, 31, 40])), int(rng.choice([1, 2])), int(rng.choice([1, 2, 4])))
+        p[W.P_ISSUE_POLICY], p[W.P_SUBPARTITIONS] = 1 + k % 2, int(rng.choice([1, 2, 4]))
+        rows.append(p)
+    rows = np.stack(rows)
+    lanes = H.run_gpu(g, rows)
+    both = H.run_gpu(g, np.concatenate([rows, _row(rng, 1, 1)[None, :]]))
+    assert np.all(lanes["status"] == 0)
+    for k in ("status", "makespan", "start", "finish", "digest", "cta_sm", "busy"):
+        assert np.array_equal(lanes[k], both[k][:rows.shape[0]]), k
