@@ -1283,16 +1283,16 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
 // Every other head issues as soon as it precedes its SM's own waiting HBM head
 // and does not pass the retirement of a CTA on its SM.  Each step of the warp
 // looks over the SMs' records, grants all it can, then issues one node on each of
-// up to 32 SMs, one per lane, and repeats that on the SMs that can go on while
-// half of them can.
+// up to 32 SMs, one per lane, and repeats that on the SMs that can go on
+// (LANE_ROUNDS).
 //
 // What bounds it: a step is some 1,000 dependent instructions of one warp at about
-// 4.4 cycles each (fixed-latency waits; 32% of the issue slots at 7 warps per SM),
+// 4.4 cycles each (fixed-latency waits; 39% of the issue slots at 7.8 warps per SM),
 // for 5 to 25 nodes where k_simulate spends 500 for one.  Measured, one GB300 at
 // 2,070 MHz, ms per batch, k_simulate then this: ws GEMM 4096x4096x2048 on 3,000
-// rows 324 and 64; FlashAttention of 54,528 nodes on 257 rows 86.5 and 17.1; decoder
-// layer of 84,672 nodes on 300 rows 128 and 32.7; GEMM 512^3 on one row 3.03 and
-// 0.55, on 64 rows 3.43 and 1.00.  73.6 warp-instructions per node on the profiling
+// rows 324 and 52-59; FlashAttention of 54,528 nodes on 257 rows 86.5 and 18; decoder
+// layer of 84,672 nodes on 300 rows 128 and 31; GEMM 512^3 on one row 3.1 and
+// 0.57, on 64 rows 3.46 and 1.02.  73.3 warp-instructions per node on the profiling
 // case (497 before).
 constexpr uint32_t LANE_SLOT_WORDS = 8;   // rdy, meta, tag, next of stream; occ, HBM occ (else servers of its class), succ
                                           // begin, latency
@@ -1548,21 +1548,24 @@ __device__ __forceinline__ void lane_refresh(const LanePt &P, uint32_t s, uint32
 // H, one that does is lost when H passes E_u.  So the record holds the SM's first
 // event (E_u, id) alone: as its first head when no waiting pick comes in the same
 // cycle, else as a candidate for the global order -- the waiting pick itself, or the
-// lower id that issues before it -- out of date once H passes its cycle, unless it is
-// the SM's only head that could issue.
+// lower id that issues before it -- out of date once H passes its cycle.  A waiting
+// pick that is its scheduler's only head moves along with H instead, out of date when
+// H reaches another scheduler's event (every grant passes the cycles of the waiting
+// picks: ws GEMM 2048x2048x1024 on 4,096 rows under GTO, 4 schedulers, 80.6 ms when
+// each of them was refreshed, 40.0 now).
 // A pick may show up late in its cycle, when a node of higher id has taken a unit of
 // the pick before it: its place in the global order is after that node.  b.w is the
 // tag of that place; of a first head, as long as H has not passed its cycle, a bound
 // on the places of the HBM heads to come.
 // The pass that finds the least key also counts the scheduler's heads: most have one,
 // which is the pick under any policy, and need no second pass (WS GEMM 2048x1024x1024
-// on 448 rows of the issue-policy axes: 12.2 ms with it, 9.8-10.4 without).
+// on 448 rows of the issue-policy axes: 12.2 ms with it, 9.8-10.3 without).
 __device__ __forceinline__ void lane_refresh_sub(const LanePt &P, uint32_t s, uint32_t H, uint4 &a, uint4 &b) {
   const uint32_t *sv = P.servers(s);
   const uint4 *sl = P.slots(s);
   uint64_t first = INF64;
-  uint32_t wait_e = INF, heads = 0;
-  bool waits = false;
+  uint32_t wait_e = INF, second = INF;  // second: least event of the other schedulers
+  bool waits = false, alone = false;
   auto key = [&](const uint4 &q) {  // INF: cannot issue
     if (q.y >= (1u << 16)) return INF;
     const uint32_t k = max(q.x, *reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(sv) + (q.y & 1023u)));
@@ -1579,7 +1582,6 @@ __device__ __forceinline__ void lane_refresh_sub(const LanePt &P, uint32_t s, ui
       tag = k != INF ? q.z : tag;
       n += k != INF ? 1u : 0u;
     }
-    heads += n;
     if (m == INF) continue;
     const uint32_t *sq = P.sub(s, u);
     const uint32_t E = max(m, sq[Q_AVAIL]), last = sq[Q_LAST];
@@ -1604,16 +1606,18 @@ __device__ __forceinline__ void lane_refresh_sub(const LanePt &P, uint32_t s, ui
     const bool w = (int32_t)tag < 0;
     if (w) wait_e = min(wait_e, E);
     const uint64_t e = pack(E, tag & ID_MASK);
+    second = min(second, (uint32_t)(max(e, first) >> 32));
     if (e < first) {
       first = e;
       waits = w;
+      alone = n == 1u;
     }
   }
   const uint32_t E = (uint32_t)(first >> 32), tag = (uint32_t)first;
   const bool cand = waits || (first != INF64 && wait_e == E);
   a = cand ? make_uint4(INF, NONE, E, tag) : make_uint4(E, tag, INF, NONE);
   b.y = cand ? INF : max(E, sv[P.off_ld]);
-  b.z = cand && heads > 1u ? E + 1u : INF;
+  b.z = cand ? max(E + 1u, waits && alone ? second : 0u) : INF;
   const uint32_t *done = P.sub(s, P.L.nsub);  // cycle of the SM's last issue, highest tag that issued in it
   b.w = E == done[0] ? max(tag, done[1]) : tag;
   P.smrec(s)[0] = a;
@@ -2055,8 +2059,8 @@ __device__ __forceinline__ uint32_t lane_grant(const DevGraph &g, const LanePt &
 }
 
 // EXT: the instance for tables with rows under the L2 model or an issue policy
-// (96 rows of the L2 study's GEMM 8.97 ms, 66.1 in k_simulate<true, false>; 448 rows
-// of the policy study 12.2 for 17.2).
+// (96 rows of the L2 study's GEMM 8.3-10 ms, 66.1 in k_simulate<true, false>; 448 rows
+// of the policy study 9.6 for 17.2).
 template <bool EXT>
 __global__ void __launch_bounds__(MAX_WPB * 32, 3)
 k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__ params, uint32_t first_point, uint32_t n_points, uint32_t flags,
