@@ -1291,8 +1291,8 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
 // for 5 to 25 nodes where k_simulate spends 500 for one.  Measured, one GB300 at
 // 2,070 MHz, ms per batch, k_simulate then this: ws GEMM 4096x4096x2048 on 3,000
 // rows 324 and 52-59; FlashAttention of 54,528 nodes on 257 rows 86.5 and 18; decoder
-// layer of 84,672 nodes on 300 rows 128 and 31; GEMM 512^3 on one row 3.1 and
-// 0.57, on 64 rows 3.46 and 1.02.  73.3 warp-instructions per node on the profiling
+// layer of 84,672 nodes on 300 rows 128 and 31; GEMM 512^3 on one row 3.0-3.3 and
+// 0.57-0.94, on 64 rows 3.46 and 1.02.  73.3 warp-instructions per node on the profiling
 // case (497 before).
 constexpr uint32_t LANE_SLOT_WORDS = 8;   // rdy, meta, tag, next of stream; occ, HBM occ (else servers of its class), succ
                                           // begin, latency
@@ -1549,23 +1549,25 @@ __device__ __forceinline__ void lane_refresh(const LanePt &P, uint32_t s, uint32
 // event (E_u, id) alone: as its first head when no waiting pick comes in the same
 // cycle, else as a candidate for the global order -- the waiting pick itself, or the
 // lower id that issues before it -- out of date once H passes its cycle.  A waiting
-// pick that is its scheduler's only head moves along with H instead, out of date when
-// H reaches another scheduler's event (every grant passes the cycles of the waiting
-// picks: ws GEMM 2048x2048x1024 on 4,096 rows under GTO, 4 schedulers, 80.6 ms when
-// each of them was refreshed, 40.0 now).
+// pick that is its scheduler's only head with a key up to E_u moves along with H
+// instead (unless it showed up late), out of date when H reaches the scheduler's next
+// key or another scheduler's event (every grant passes the cycles of the waiting picks:
+// ws GEMM 2048x2048x1024 on 4,096 rows under GTO, 4 schedulers, 80.6 ms when each of
+// them was refreshed, 40.0 now).
 // A pick may show up late in its cycle, when a node of higher id has taken a unit of
 // the pick before it: its place in the global order is after that node.  b.w is the
 // tag of that place; of a first head, as long as H has not passed its cycle, a bound
 // on the places of the HBM heads to come.
-// The pass that finds the least key also counts the scheduler's heads: most have one,
-// which is the pick under any policy, and need no second pass (WS GEMM 2048x1024x1024
-// on 448 rows of the issue-policy axes: 12.2 ms with it, 9.8-10.3 without).
+// The pass that finds the least key also finds the second least: beyond E_u, as mostly,
+// the first's head is the pick under any policy, and there is no second pass (WS GEMM
+// 2048x1024x1024 on 448 rows of the issue-policy axes: 12.2 ms with it, 6.0-7.1 now).
 __device__ __forceinline__ void lane_refresh_sub(const LanePt &P, uint32_t s, uint32_t H, uint4 &a, uint4 &b) {
   const uint32_t *sv = P.servers(s);
   const uint4 *sl = P.slots(s);
   uint64_t first = INF64;
   uint32_t wait_e = INF, second = INF;  // second: least event of the other schedulers
-  bool waits = false, alone = false;
+  uint32_t next_key = INF;               // second least key of the first event's scheduler
+  bool waits = false;
   auto key = [&](const uint4 &q) {  // INF: cannot issue
     if (q.y >= (1u << 16)) return INF;
     const uint32_t k = max(q.x, *reinterpret_cast<const uint32_t *>(reinterpret_cast<const char *>(sv) + (q.y & 1023u)));
@@ -1573,21 +1575,21 @@ __device__ __forceinline__ void lane_refresh_sub(const LanePt &P, uint32_t s, ui
   };
 #pragma unroll 1
   for (uint32_t u = 0; u < P.L.nsub; u++) {
-    uint32_t m = INF, tag = 0, n = 0;
+    uint32_t m = INF, m2 = INF, tag = 0;
 #pragma unroll 2
     for (uint32_t l = u; l < P.L.per; l += P.L.nsub) {
       const uint4 q = sl[2 * l];
       const uint32_t k = key(q);
+      tag = k < m ? q.z : tag;
+      m2 = min(m2, max(m, k));
       m = min(m, k);
-      tag = k != INF ? q.z : tag;
-      n += k != INF ? 1u : 0u;
     }
     if (m == INF) continue;
     const uint32_t *sq = P.sub(s, u);
     const uint32_t E = max(m, sq[Q_AVAIL]), last = sq[Q_LAST];
     uint32_t best = INF;
 #pragma unroll 2
-    for (uint32_t l = u; n > 1u && l < P.L.per; l += P.L.nsub) {  // among several heads the policy picks
+    for (uint32_t l = u; m2 <= E && l < P.L.per; l += P.L.nsub) {  // among several heads up to E the policy picks
       const uint4 q = sl[2 * l];
       if (key(q) > E) continue;
       uint32_t order;
@@ -1610,16 +1612,16 @@ __device__ __forceinline__ void lane_refresh_sub(const LanePt &P, uint32_t s, ui
     if (e < first) {
       first = e;
       waits = w;
-      alone = n == 1u;
+      next_key = m2;
     }
   }
   const uint32_t E = (uint32_t)(first >> 32), tag = (uint32_t)first;
   const bool cand = waits || (first != INF64 && wait_e == E);
   a = cand ? make_uint4(INF, NONE, E, tag) : make_uint4(E, tag, INF, NONE);
   b.y = cand ? INF : max(E, sv[P.off_ld]);
-  b.z = cand ? max(E + 1u, waits && alone ? second : 0u) : INF;
   const uint32_t *done = P.sub(s, P.L.nsub);  // cycle of the SM's last issue, highest tag that issued in it
   b.w = E == done[0] ? max(tag, done[1]) : tag;
+  b.z = cand ? max(E + 1u, waits && b.w == tag ? min(second, next_key) : 0u) : INF;
   P.smrec(s)[0] = a;
   P.smrec(s)[1] = b;
 }
@@ -2059,8 +2061,8 @@ __device__ __forceinline__ uint32_t lane_grant(const DevGraph &g, const LanePt &
 }
 
 // EXT: the instance for tables with rows under the L2 model or an issue policy
-// (96 rows of the L2 study's GEMM 8.3-10 ms, 66.1 in k_simulate<true, false>; 448 rows
-// of the policy study 9.6 for 17.2).
+// (96 rows of the L2 study's GEMM 8.3-12 ms, 66.1 in k_simulate<true, false>; 448 rows
+// of the policy study 6.0-7.1 for 17.2).
 template <bool EXT>
 __global__ void __launch_bounds__(MAX_WPB * 32, 3)
 k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__ params, uint32_t first_point, uint32_t n_points, uint32_t flags,
