@@ -2000,6 +2000,7 @@ __device__ __forceinline__ uint32_t lane_grant(const DevGraph &g, const LanePt &
         X.loads += tile ? ti & 1u : 0u;
       }
     }
+    if (EXT && X.cap) __syncwarp();  // the list is in shared memory and another lane may win the next turn
     ho = __reduce_max_sync(FULL, win ? ho : 0u);
     const bool takes = !EXT || ho != NONE;
     if (takes && (uint64_t)t + ho > 0x7FFFFFFFull) return NONE;
