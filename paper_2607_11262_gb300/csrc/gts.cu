@@ -799,7 +799,9 @@ __device__ __forceinline__ void put_constants(uint32_t *sp, const int32_t *prm, 
     *reinterpret_cast<uint64_t *>(sp + O_MAG + 12) = div_const((uint32_t)prm[GTS_P_L2_BPC]);
   } else if (lane == 30) {  // LOAD base with the L2 model: hit, miss
     sp[O_L2B] = (uint32_t)prm[GTS_P_TMA_LAT] + (uint32_t)prm[GTS_P_L2_LAT];
-    sp[O_L2B + 1] = (uint32_t)prm[GTS_P_TMA_LAT] + (uint32_t)prm[GTS_P_L2_LAT] + (uint32_t)prm[GTS_P_DRAM_LAT];
+    // three latencies may pass 2^32; 2^31 overflows whatever the rest of the node adds
+    const uint64_t miss = (uint64_t)sp[O_L2B] + (uint32_t)prm[GTS_P_DRAM_LAT];
+    sp[O_L2B + 1] = miss > 0x80000000ull ? 0x80000000u : (uint32_t)miss;
   }
   if (lane < 8) {  // base latency per type: LOAD, SMEM, MMA, EW, STORE, BAR, NOP
     uint32_t bl = 0;

@@ -13,15 +13,6 @@ from tests import tinygraphs as TG
 from tests import warp_emulation as E
 
 
-@pytest.fixture(scope="module")
-def warp(tmp_path_factory):
-    path = str(tmp_path_factory.mktemp("warp"))
-    exe = E.build(path)
-    if exe is None:
-        pytest.skip("no g++ with the thread sanitizer")
-    return exe, path
-
-
 def races(report):
     """The reports, less those of one statement by which several lanes store the same value."""
     out = []
