@@ -245,7 +245,7 @@ __host__ __device__ inline bool make_layout(const int32_t *p, uint32_t CG, uint3
   L.csms = (uint32_t)p[GTS_P_CLUSTER_SMS];
   L.cap_noc = (class_mask & CM_NOC) ? (uint32_t)p[GTS_P_CAP_NOC] : 0u;
   L.o_ns = (uint32_t)w;  // NoC servers per SM group
-  if (L.cap_noc) w += (uint64_t)((L.NS + L.csms - 1) / L.csms) * (L.cap_noc + 1);  // and their first free cycle
+  if (L.cap_noc) w += (uint64_t)((L.NS + L.csms - 1) / L.csms) * L.cap_noc;
   w = (w + 3) & ~(uint64_t)3;  // 16-byte multiple
   if (w * 4 > MAX_SMEM_BYTES) return false;
   L.words = (uint32_t)w;
@@ -379,9 +379,8 @@ __device__ __forceinline__ uint32_t slot_key(const Pt &P, uint32_t i, uint32_t s
     uint32_t a = sv[0];
     for (uint32_t q = 1; q < cap; q++) a = min(a, sv[q]);
     k = max(k, a);
-    if (NOC && cls == RC_DSM) {  // and a NoC server of the SM's group
-      k = max(k, P.sp[P.L.o_ns + div16(sm, P.mCsms) * (P.L.cap_noc + 1u) + P.L.cap_noc]);
-    }
+    if (NOC && cls == RC_DSM)  // and a NoC server of the SM's group, whose first free one comes first
+      k = max(k, P.sp[P.L.o_ns + div16(sm, P.mCsms) * P.L.cap_noc]);
   }
   return k;
 }
@@ -920,7 +919,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
     for (uint32_t k = lane; k < P.L.NS * P.L.SC; k += 32) sp[P.L.o_sv + k] = 0u;
     for (uint32_t k = lane; k < P.L.cap_hbm; k += 32) sp[P.L.o_hs + k] = 0u;
     if (NOC && P.L.cap_noc)
-      for (uint32_t k = lane; k < ((P.L.NS + P.L.csms - 1) / P.L.csms) * (P.L.cap_noc + 1u); k += 32) sp[P.L.o_ns + k] = 0u;
+      for (uint32_t k = lane; k < ((P.L.NS + P.L.csms - 1) / P.L.csms) * P.L.cap_noc; k += 32) sp[P.L.o_ns + k] = 0u;
     for (uint32_t k = lane; k < P.L.NS * P.L.nsub; k += 32) {
       sp[P.L.o_sub + k * SUB_WORDS + Q_AVAIL] = 0u;
       sp[P.L.o_sub + k * SUB_WORDS + Q_LAST] = NONE;
@@ -1029,15 +1028,18 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
       }
       bool noc_touch = false;  // the last free NoC server of the SM's group was taken
       if (NOC && cls == RC_DSM) {
-        uint32_t *ns = sp + P.L.o_ns + div16(sm, P.mCsms) * (P.L.cap_noc + 1u);
-        uint32_t v = (uint32_t)lane < P.L.cap_noc ? ns[lane] : INF;
-        const uint32_t bal = __ballot_sync(FULL, v <= t);
-        if (lane == __ffs(bal) - 1) ns[lane] = v = t + nocc;
-        v = __reduce_min_sync(FULL, v);
-        if (lane == 0) ns[P.L.cap_noc] = v;
-        // with a server still free at t, no other head's key moved; the group's first free cycle is kept, because
-        // reading all servers per key and rekeying the group at every issue took 35% of the fused attention's time
-        noc_touch = P.L.csms > 1u && v > t;
+        // the node takes the group's first free server, at the front, and the next one free changes places with it: with
+        // one still free at t no other head's key moved.  (Reading all servers per key and rekeying the group at every
+        // issue took 35% of the fused attention's time.)
+        uint32_t *ns = sp + P.L.o_ns + div16(sm, P.mCsms) * P.L.cap_noc;
+        const uint32_t v = lane == 0 ? t + nocc : (uint32_t)lane < P.L.cap_noc ? ns[lane] : INF;
+        const uint32_t next = __reduce_min_sync(FULL, v);
+        const uint32_t at = __ffs(__ballot_sync(FULL, v == next)) - 1;
+        if (lane == 0) {
+          ns[at] = v;
+          ns[0] = next;
+        }
+        noc_touch = P.L.csms > 1u && next > t;
       }
       if (EXT && P.L.nsub && lane == 0) {  // the issuing scheduler: one issue per cycle, remember the slot
         const uint32_t l = i - sm * P.L.per;
