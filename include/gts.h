@@ -371,6 +371,16 @@ gts_status gts_simulate_batch(gts_graph *graph, gts_params *params,
                               void *d_scratch, size_t scratch_bytes,
                               void *stream, gts_results **out);
 
+/* Which kernel gts_simulate_batch launches for these points, given scratch for
+ * every resident warp: GTS_PLAN_* bits, or a negative gts_status.  No bit: the
+ * general kernel, one node per step, for lowest-id rows.  Results do not depend
+ * on it; for tests and measurements.  Errors: INVALID_ARG, CUDA. */
+#define GTS_PLAN_LANES    1   /* the lane-parallel kernel: one simulated SM per lane */
+#define GTS_PLAN_EXTENDED 2   /* ... instance for issue policies and the L2 model */
+#define GTS_PLAN_NOC      4   /* ... and the NoC of DSMEM nodes */
+#define GTS_PLAN_PADDED   8   /* lanes: an SM's warp slots padded to a multiple of four */
+int32_t gts_batch_plan(const gts_graph *graph, const gts_params *params, uint32_t first_point, uint32_t n_points);
+
 /* Waits for the batch and copies its per-point arrays -- the kernel makespan
  * of each design point (Section 5.1: the cycle the last node completes), its
  * status and digest -- to the host (any h_* may be NULL; n_points <= the

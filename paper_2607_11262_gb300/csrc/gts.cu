@@ -1321,7 +1321,8 @@ constexpr uint32_t EXHAUSTED = 0xFFFF0000u;
 constexpr uint32_t LANE_DEG_BIG = 7;
 // L2 list in shared memory: head, tail, bytes in use; per tile 16-bit links to the more and the less recent tile
 // (L2_NIL: none; the pair L2_OUT: not listed) and its bytes
-constexpr uint32_t L2_NIL = 0xFFFFu, L2_OUT = 0xFFFEFFFEu, L2_MAX_TILES = 0xFFFDu;
+constexpr uint32_t L2_NIL = 0xFFFFu, L2_OUT = 0xFFFEFFFEu;
+static_assert(MAX_SMEM_BYTES / 8 < 0xFFFEu, "tile ids of a list that fits shared memory (two words each) stay below the marks");
 
 struct LaneLayout {
   uint32_t Scta, NS, SC, per, per4, cap_hbm, nsub;
@@ -1332,7 +1333,7 @@ struct LaneLayout {
 // and are read as they lie; without, the last group of four repeats a slot.
 // `tiles`: entries of the row's L2 list, 0 without the L2 model.
 __host__ __device__ inline bool make_lane_layout(const Layout &B, bool pad, uint32_t tiles, LaneLayout &L) {
-  if (tiles > L2_MAX_TILES || B.cap_noc || B.NS > LANE_MAX_SMS || B.per > LANE_MAX_SLOTS) return false;
+  if (B.cap_noc || B.NS > LANE_MAX_SMS || B.per > LANE_MAX_SLOTS) return false;
   L.nsub = B.nsub;
   L.Scta = B.Scta; L.NS = B.NS; L.SC = B.SC + 1; L.per = B.per; L.per4 = pad ? (B.per + 3u) & ~3u : B.per; L.cap_hbm = B.cap_hbm;
   uint64_t w = O_DYN;
@@ -3213,6 +3214,18 @@ size_t gts_scratch_bytes(const gts_graph *g, const gts_params *P, uint32_t flags
   Plan pl;
   if (plan_launch(g, P, 0, P->n_points, flags, 0, false, pl) != GTS_OK) return 0;
   return GTS_SCRATCH_HEADER_BYTES + (size_t)pl.warps * scratch_row_bytes(g);
+}
+
+int32_t gts_batch_plan(const gts_graph *g, const gts_params *P, uint32_t first_point, uint32_t n_points) {
+  clear_error();
+  if (!g || !P || P->graph != g) return fail(GTS_ERR_INVALID_ARG, "null or mismatched graph / params");
+  if ((uint64_t)first_point + n_points > P->n_points) return fail(GTS_ERR_INVALID_ARG, "point range outside the table");
+  if (!n_points) return 0;
+  Plan pl;
+  const gts_status st = plan_launch(g, P, first_point, n_points, 0, 0, false, pl);
+  if (st != GTS_OK) return st;
+  return (pl.lanes ? GTS_PLAN_LANES | (pl.pad ? GTS_PLAN_PADDED : 0) : 0) | (pl.sched || pl.noc ? GTS_PLAN_EXTENDED : 0) |
+         (pl.noc ? GTS_PLAN_NOC : 0);
 }
 
 gts_status gts_simulate_batch(gts_graph *g, gts_params *P, uint32_t first_point, uint32_t n_points, uint32_t flags,

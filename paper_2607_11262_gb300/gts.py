@@ -35,6 +35,8 @@ GTS_WANT_CTA_SM = 4
 GTS_WANT_BUSY = 8
 GTS_SCRATCH_CLEAN = 16
 
+GTS_PLAN_LANES, GTS_PLAN_EXTENDED, GTS_PLAN_NOC, GTS_PLAN_PADDED = 1, 2, 4, 8
+
 GTS_BUSY_CLASSES = 9
 (GTS_BUSY_TENSOR, GTS_BUSY_TMA, GTS_BUSY_LSU, GTS_BUSY_ALU, GTS_BUSY_BAR, GTS_BUSY_HBM, GTS_BUSY_NOC,
  GTS_BUSY_L2_HITS, GTS_BUSY_L2_LOADS) = range(9)
@@ -48,7 +50,7 @@ GTS_SCRATCH_HEADER_BYTES = 16
 
 EXPORTS = ("gts_graph_workspace_bytes", "gts_graph_create", "gts_graph_destroy", "gts_template_workspace_bytes",
            "gts_graph_create_templated", "gts_params_upload", "gts_params_set_order",
-           "gts_params_destroy", "gts_row_nodes", "gts_row_ctas", "gts_scratch_bytes", "gts_simulate_batch",
+           "gts_params_destroy", "gts_row_nodes", "gts_row_ctas", "gts_scratch_bytes", "gts_batch_plan", "gts_simulate_batch",
            "gts_read_results", "gts_results_destroy", "gts_simulate_batch_noalloc", "gts_last_error")
 
 
@@ -115,6 +117,8 @@ def load():
     lib.gts_row_ctas.restype = u32
     lib.gts_scratch_bytes.argtypes = [vp, vp, u32]
     lib.gts_scratch_bytes.restype = sz
+    lib.gts_batch_plan.argtypes = [vp, vp, u32, u32]
+    lib.gts_batch_plan.restype = i32
     lib.gts_simulate_batch.argtypes = [vp, vp, u32, u32, u32, vp, vp, vp, vp, vp, vp, vp, vp, sz, vp, pp]
     lib.gts_simulate_batch.restype = i32
     lib.gts_read_results.argtypes = [vp, vp, vp, vp, u32]
@@ -184,6 +188,13 @@ def gts_row_ctas(graph):
 
 def gts_scratch_bytes(graph, params, flags):
     return int(load().gts_scratch_bytes(graph, params, flags))
+
+
+def gts_batch_plan(graph, params, first_point, n_points):
+    """GTS_PLAN_* bits of the kernel gts_simulate_batch launches for these points."""
+    plan = int(load().gts_batch_plan(graph, params, first_point, n_points))
+    _check(min(plan, 0))
+    return plan
 
 
 def gts_simulate_batch(graph, params, first_point, n_points, flags, d_start, d_finish, d_makespan, d_status,

@@ -52,7 +52,8 @@ def run_gpu(graph, params, flags=None, first_point=0, n_points=None):
     dp = gts.DeviceParams(dg, params)
     out = gts.simulate(dg, dp, first_point=first_point, n_points=n_points, flags=flags)
     torch.cuda.synchronize()
-    res = {"status": out.status.cpu().numpy(), "makespan": out.makespan.cpu().numpy()}
+    res = {"status": out.status.cpu().numpy(), "makespan": out.makespan.cpu().numpy(),
+           "plan": gts.gts_batch_plan(dg.handle, dp.handle, first_point, out.status.numel())}
     if out.start is not None:
         res["start"] = out.start.cpu().numpy()
         res["finish"] = out.finish.cpu().numpy()

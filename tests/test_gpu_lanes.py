@@ -4,7 +4,8 @@ are in CTA order with no edge between CTAs: against the oracle where its tiles
 end (SMs per lane round, slots read four at a time, the inline successors,
 servers kept in registers up to four, L2 lists in shared memory), and against
 the general instance, which the same rows run in when the batch also holds a row
-of one SM.  Integer results, compared bit for bit."""
+of 33 warp slots on an SM.  Each test states the kernel it means (H.run_gpu gives
+the plan).  Integer results, compared bit for bit."""
 import numpy as np
 import pytest
 
@@ -47,7 +48,11 @@ def _row(rng, sms, cps, cap_hbm=1, cap_tma=1, cap_lsu=4):
     return p
 
 
-def _check(g, rows, res):
+LANES = 1   # GTS_PLAN_LANES
+
+
+def _check(g, rows, res, lanes=True):
+    assert bool(res["plan"] & LANES) == lanes, res["plan"]
     for q in range(rows.shape[0]):
         H.assert_point_equal(g, rows[q], res, q, oracle_run.simulate(g, rows[q]))
 
@@ -59,7 +64,7 @@ def test_sm_counts(sms):
     for mix in range(4):
         g = _graph(rng, 700, 170, 2, mix, kernels=mix == 3)
         rows = np.stack([_row(rng, sms, 1, cap_hbm=c) for c in (1, 1, 3)])
-        _check(g, rows, H.run_gpu(g, rows))
+        _check(g, rows, H.run_gpu(g, rows), lanes=sms <= 160)
 
 
 @pytest.mark.parametrize("warps,cps", [(1, 1), (3, 1), (4, 1), (5, 1), (3, 3), (8, 4), (11, 3)])
@@ -68,7 +73,7 @@ def test_slots_per_sm(warps, cps):
     rng = np.random.default_rng(7100 + warps * cps)
     g = _graph(rng, 300, 20, warps, 0, kernels=True)
     rows = np.stack([_row(rng, s, cps) for s in (2, 3, 5)])
-    _check(g, rows, H.run_gpu(g, rows))
+    _check(g, rows, H.run_gpu(g, rows), lanes=warps * cps <= 32)
 
 
 @pytest.mark.parametrize("caps", [(1, 1, 1), (2, 2, 2), (4, 4, 4), (1, 5, 5), (32, 32, 32)])
@@ -95,9 +100,27 @@ def test_successor_counts(fan):
     _check(g, rows, H.run_gpu(g, rows))
 
 
+@pytest.mark.parametrize("mix", range(4))
+def test_nodes_without_work(mix):
+    """Nodes that hold their unit for no cycle; their latency is positive."""
+    rng = np.random.default_rng(7350 + mix)
+    g = _graph(rng, 300, 40, 3, mix, kernels=mix == 1)
+    g.work[rng.random(g.n_nodes) < 0.4] = 0
+    rows = np.stack([_row(rng, s, c, h) for s, c, h in ((2, 1, 1), (5, 2, 2), (33, 1, 1), (40, 1, 3))])
+    _check(g, rows, H.run_gpu(g, rows))
+
+
+def _beside_33_slots(rng, g, rows):
+    """The rows of a batch that runs in the general kernel because of one more row."""
+    wide = _row(rng, 2, -(-33 // g.warps_per_cta))
+    res = H.run_gpu(g, np.concatenate([rows, wide[None, :]]))
+    assert not res["plan"] & LANES
+    return res
+
+
 @pytest.mark.parametrize("seed", range(6))
 def test_agrees_with_the_general_instance(seed):
-    """Rows over all forms the rule takes, alone and beside a row of one SM."""
+    """Rows over all forms the rule takes, alone and beside a row of 33 slots per SM."""
     rng = np.random.default_rng(7400 + seed)
     g = _graph(rng, 400, int(rng.integers(20, 60)), int(rng.integers(1, 7)), seed % 4, kernels=seed % 2 == 1,
                max_work=[2, 6, 60][seed % 3], p_issue=[0.0, 0.3, 0.9][seed % 3])
@@ -108,7 +131,8 @@ def test_agrees_with_the_general_instance(seed):
     rows[7, W.P_TMA_BPC] = 0                    # refused
     rows[11, W.P_DRAM_LAT] = 2**31 - 40         # overflows
     lanes = H.run_gpu(g, rows)
-    both = H.run_gpu(g, np.concatenate([rows, _row(rng, 1, 1)[None, :]]))
+    assert lanes["plan"] & LANES
+    both = _beside_33_slots(rng, g, rows)
     n = rows.shape[0]
     for k in ("status", "makespan"):
         assert np.array_equal(lanes[k], both[k][:n]), k
@@ -139,6 +163,7 @@ def test_points_taken_by_cost_class():
     dg = gts.DeviceGraph(w.graph)
     dp = gts.DeviceParams(dg, w.params)
     row = (dg.row_nodes + 1) // 2 * 16
+    assert gts.gts_batch_plan(dg.handle, dp.handle, 0, 120) & LANES
     few = torch.zeros(gts.GTS_SCRATCH_HEADER_BYTES + 7 * row, dtype=torch.uint8, device="cuda")
     full = gts.simulate(dg, dp, flags=gts.GTS_WANT_DIGEST)
     part = gts.simulate(dg, dp, first_point=11, n_points=90, flags=gts.GTS_WANT_DIGEST | gts.GTS_SCRATCH_CLEAN,
@@ -161,8 +186,10 @@ def test_dense_slots_agree_with_padded_ones(k):
     dg = gts.DeviceGraph(g)
     dp = gts.DeviceParams(dg, p)
     flags = gts.GTS_WANT_DIGEST | gts.GTS_WANT_BUSY
+    assert gts.gts_batch_plan(dg.handle, dp.handle, 0, 3000) == LANES
     whole = gts.simulate(dg, dp, flags=flags)
     for lo in range(0, 3000, 600):
+        assert gts.gts_batch_plan(dg.handle, dp.handle, lo, 600) == LANES | gts.GTS_PLAN_PADDED
         part = gts.simulate(dg, dp, first_point=lo, n_points=600, flags=flags)
         torch.cuda.synchronize()
         for f in ("status", "makespan", "digest", "busy"):
@@ -176,9 +203,9 @@ def _with_l2(rng, p, tiles_bytes):
     return p
 
 
-@pytest.mark.parametrize("tiles", [1, 7, 64, 3000, 65533, 65534])
+@pytest.mark.parametrize("tiles", [1, 7, 64, 3000])
 def test_l2_lists(tiles):
-    """The L2 list in shared memory, up to its largest tile count (and one more, which the general instance runs)."""
+    """The L2 list in shared memory."""
     rng = np.random.default_rng(7600 + tiles)
     for mix in (0, 2):
         g = _graph(rng, 220, 24, 3, mix, kernels=mix == 2)
@@ -188,6 +215,20 @@ def test_l2_lists(tiles):
         rows = [_row(rng, int(rng.choice([2, 5, 40])), int(rng.integers(1, 3)), int(rng.integers(1, 3))) for _ in range(5)]
         rows = np.stack([rows[0]] + [_with_l2(rng, p, [1, 6, 30, 10**6]) for p in rows[1:]])
         _check(g, rows, H.run_gpu(g, rows))
+
+
+@pytest.mark.parametrize("tiles", [28906, 28907])
+def test_l2_list_limit(tiles):
+    """The longest list of a point with two SMs of three warps (299 other words, 58,112 in all), and one more tile,
+    which the general instance runs."""
+    rng = np.random.default_rng(7650)
+    g = _graph(rng, 400, 30, 3, 0)
+    g.tile = rng.integers(tiles - 90, tiles, g.n_nodes).astype(np.uint32)
+    g.tile[::6] = W.NO_TILE
+    g.n_tiles = tiles
+    rows = np.stack([_with_l2(rng, _row(rng, 2, 1), [1, 30, 200, 10**6]) for _ in range(4)])
+    rows[:, W.P_CAP_TENSOR:W.P_CAP_HBM + 1] = 1
+    _check(g, rows, H.run_gpu(g, rows), lanes=tiles == 28906)
 
 
 @pytest.mark.parametrize("schedulers", [1, 2, 3, 4, 7, 32])
@@ -221,7 +262,8 @@ def test_policies_agree_with_the_general_instance(seed):
         rows.append(p)
     rows = np.stack(rows)
     lanes = H.run_gpu(g, rows)
-    both = H.run_gpu(g, np.concatenate([rows, _row(rng, 1, 1)[None, :]]))
+    assert lanes["plan"] & LANES
+    both = _beside_33_slots(rng, g, rows)
     assert np.all(lanes["status"] == 0)
     for k in ("status", "makespan", "start", "finish", "digest", "cta_sm", "busy"):
         assert np.array_equal(lanes[k], both[k][:rows.shape[0]]), k
