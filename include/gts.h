@@ -379,6 +379,7 @@ gts_status gts_simulate_batch(gts_graph *graph, gts_params *params,
 #define GTS_PLAN_EXTENDED 2   /* ... instance for issue policies and the L2 model */
 #define GTS_PLAN_NOC      4   /* ... and the NoC of DSMEM nodes */
 #define GTS_PLAN_PADDED   8   /* lanes: an SM's warp slots padded to a multiple of four */
+#define GTS_PLAN_SPLIT    16  /* general kernel: an SM's single HBM head kept apart (SMs of fewer than 8 warp slots) */
 int32_t gts_batch_plan(const gts_graph *graph, const gts_params *params, uint32_t first_point, uint32_t n_points);
 
 /* Waits for the batch and copies its per-point arrays -- the kernel makespan

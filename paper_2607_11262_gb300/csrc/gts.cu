@@ -31,7 +31,10 @@
 //    minimum (one pass, two independent reductions, for SMs of <= 16 slots);
 //    when H moves, the SMs whose HBM heads it overtakes are recomputed (each
 //    lane its own SMs, or one SM at a time a slot per lane when SMs hold 8
-//    slots or more).  A release into a head of another
+//    slots or more).  When every SM has fewer than 8 slots, an SM whose only
+//    issuable HBM head is one keeps that head apart in its summary and takes
+//    its effective cycle max(key, H) when the summary is read, so such SMs
+//    need no recomputation when H moves.  A release that readies a head of another
 //    CTA recomputes every SM (the extended instance: the SMs it reached).
 //  * The issue itself runs in every lane on broadcast values (no divergence);
 //    only global atomics and scratch-counter reads are lane 0's.
@@ -644,6 +647,199 @@ __device__ __forceinline__ void refresh_owner(const Pt &P, uint32_t owner, int l
   if ((uint32_t)lane == owner) { b = best; bsl = slot; }
 }
 
+// ---- split SM records (plain instance, SMs of fewer than 8 slots).  An SM
+// with exactly one issuable HBM head keeps it apart from its other heads:
+// words 0-1 hold the best NON-HBM head (effective cycle, id), word 2 that
+// head's slot | the HBM head's slot << 16, word 3 the HBM head's key.  The HBM
+// head's effective cycle max(key, H) is taken where the record is read, so a
+// horizon move needs no rescan of such an SM.  Any other SM keeps the whole
+// record (best head at the horizon of its last refresh, slot | SPLIT_NONE,
+// least HBM key) and is rescanned when H passes that key.  Batches of 3 slots per
+// SM that the lanes do not take, ms without and with it: ws GEMM 2048x2048x1024 with
+// one NOP of no latency on 300 rows 20.6 and 18.3, 3,000 rows 43.7 and 39.4; ws GEMM
+// 4096x4096x512 on 192 SMs 47.5 and 40.6; 1,536 rows of one-SM pipelines 1.97 and
+// 1.86.  Without edges between CTAs, so the instance has no code for them; where they
+// are (4,000-node graphs of 3 and 4 slots) it was 1-4% slower than whole records.
+constexpr uint32_t SPLIT_NONE = 0xFFFF0000u;
+constexpr uint32_t SPLIT_SLOTS = 8;
+
+__device__ __forceinline__ void put_split_rec(const Pt &P, uint32_t s, uint64_t nh, uint32_t nhslot, uint64_t all,
+                                              uint32_t allslot, uint32_t hcnt, uint32_t hslot, uint32_t hmin) {
+  uint32_t *o = P.smrec(s);
+  const bool one = hcnt == 1u;
+  const uint64_t v = one ? nh : all;
+  o[0] = (uint32_t)v;
+  o[1] = (uint32_t)(v >> 32);
+  o[2] = (v == INF64 ? 0u : (one ? nhslot : allslot)) | (one ? hslot << 16 : SPLIT_NONE);
+  o[3] = hmin;
+}
+
+// Best (effective cycle << 32 | id) of SM s at horizon H, and its slot.
+__device__ __forceinline__ uint64_t split_sm_best(const Pt &P, uint32_t s, uint32_t H, uint32_t &slot) {
+  const uint32_t *o = P.smrec(s);
+  const uint2 a = *reinterpret_cast<const uint2 *>(o);
+  const uint2 c = *reinterpret_cast<const uint2 *>(o + 2);
+  uint64_t v = pack(a.y, a.x);
+  slot = c.x & 0xFFFFu;
+  if ((c.x >> 16) != 0xFFFFu) {
+    const uint64_t hv = pack(max(c.y, H), P.slot(c.x >> 16)[F_HID] & ID_MASK);
+    if (hv < v) {
+      v = hv;
+      slot = c.x >> 16;
+    }
+  }
+  return v;
+}
+
+// Warp-parallel refresh of SM s (all its slots in one round of lanes).
+__device__ __forceinline__ void split_refresh_sm(const Pt &P, uint32_t s, uint32_t t, uint32_t H, int lane) {
+  const uint32_t i0 = s * P.L.per, i = i0 + lane;
+  uint64_t val = INF64;
+  uint32_t hk = INF;
+  bool hf = false;
+  if (lane < (int)P.L.per && i < P.L.S) {
+    const uint32_t k = slot_key<false>(P, i, s, t);
+    const uint32_t h = P.slot(i)[F_HID];
+    if (k != INF) {
+      hf = (h & HBM_BIT) != 0u;
+      val = pack(hf ? max(k, H) : k, h & ID_MASK);
+      if (hf) hk = k;
+    }
+  }
+  const uint32_t hcnt = __popc(__ballot_sync(FULL, hf));
+  uint32_t who;
+  const uint64_t m = warp_min64(hcnt == 1u && hf ? INF64 : val, who);
+  const uint32_t hmin = __reduce_min_sync(FULL, hk);
+  if (hcnt == 1u ? hf : lane == 0) put_split_rec(P, s, m, i0 + who, m, i0 + who, hcnt, i, hmin);
+  __syncwarp();
+}
+
+// Warp-parallel, as refresh_sm_owner: SM s's record and the owner lane's best
+// (b, bsl) from two independent reductions over the same values.
+__device__ __forceinline__ void split_refresh_sm_owner(const Pt &P, uint32_t s, uint32_t t, uint32_t H, int lane,
+                                                       uint64_t &b, uint32_t &bsl) {
+  const uint32_t per = P.L.per, i0 = s * per, owner = s & 31u, l = (uint32_t)lane;
+  uint64_t vs = INF64, vo = INF64;
+  uint32_t hk = INF, so = 0;
+  bool hf = false;
+  if (l < per && i0 + l < P.L.S) {
+    const uint32_t k = slot_key<false>(P, i0 + l, s, t);
+    if (k != INF) {
+      const uint32_t h = P.slot(i0 + l)[F_HID];
+      hf = (h & HBM_BIT) != 0u;
+      vs = pack(hf ? max(k, H) : k, h & ID_MASK);
+      if (hf) hk = k;
+    }
+  } else if (l >= 16u) {
+    const uint32_t sj = owner + 32u * (l - 16u);
+    if (sj < P.L.NS && sj != s) vo = split_sm_best(P, sj, H, so);
+  }
+  const bool one = __popc(__ballot_sync(FULL, hf)) == 1u;
+  uint32_t wa, wb;
+  const uint64_t ma = warp_min64(one && hf ? INF64 : vs, wa);
+  const uint64_t mb = warp_min64(vs < vo ? vs : vo, wb);
+  const uint32_t hmin = __reduce_min_sync(FULL, hk);
+  const uint32_t sb = __shfl_sync(FULL, l < 16u ? i0 + l : so, wb);
+  if (one ? hf : lane == 0) {
+    uint32_t *o = P.smrec(s);
+    o[0] = (uint32_t)ma;
+    o[1] = (uint32_t)(ma >> 32);
+    o[2] = (ma == INF64 ? 0u : i0 + wa) | (one ? (i0 + l) << 16 : SPLIT_NONE);
+    o[3] = hmin;
+  }
+  if (l == owner) {
+    b = mb;
+    bsl = mb == INF64 ? 0u : sb;
+  }
+  __syncwarp();
+}
+
+// One lane: recompute the record of SM s at cycle t and horizon H.
+__device__ __forceinline__ void split_rescan_sm_lane(const Pt &P, uint32_t s, uint32_t t, uint32_t H) {
+  const uint32_t i0 = s * P.L.per, i1 = min(i0 + P.L.per, P.L.S);
+  uint64_t best = INF64, nbest = INF64;
+  uint32_t bsl = 0, nsl = 0, hmin = INF, hcnt = 0, hslot = 0;
+  for (uint32_t i = i0; i < i1; i++) {
+    const uint32_t k = slot_key<false>(P, i, s, t);
+    if (k == INF) continue;
+    const uint32_t h = P.slot(i)[F_HID];
+    const bool hb = (h & HBM_BIT) != 0u;
+    const uint64_t val = pack(hb ? max(k, H) : k, h & ID_MASK);
+    if (hb) {
+      hmin = min(hmin, k);
+      hcnt++;
+      hslot = i;
+    } else if (val < nbest) {
+      nbest = val;
+      nsl = i;
+    }
+    if (val < best) { best = val; bsl = i; }
+  }
+  put_split_rec(P, s, nbest, nsl, best, bsl, hcnt, hslot, hmin);
+}
+
+__device__ __forceinline__ uint64_t split_lane_best(const Pt &P, int lane, uint32_t H, uint32_t &slot) {
+  uint64_t b = INF64;
+  slot = 0;
+  for (uint32_t s = lane; s < P.L.NS; s += 32) {
+    uint32_t sl;
+    const uint64_t v = split_sm_best(P, s, H, sl);
+    if (v < b) { b = v; slot = sl; }
+  }
+  return b;
+}
+
+__device__ __forceinline__ void split_refresh_owner(const Pt &P, uint32_t owner, int lane, uint32_t H, uint64_t &b,
+                                                    uint32_t &bsl) {
+  uint64_t best = INF64;
+  uint32_t slot = 0;
+  for (uint32_t base = owner; base < P.L.NS; base += 32 * 32) {
+    const uint32_t s = base + 32u * lane;
+    uint64_t val = INF64;
+    uint32_t sl = 0;
+    if (s < P.L.NS) val = split_sm_best(P, s, H, sl);
+    uint32_t who;
+    const uint64_t m = warp_min64(val, who);
+    const uint32_t ws = __shfl_sync(FULL, sl, who);
+    if (m < best) { best = m; slot = ws; }
+  }
+  if ((uint32_t)lane == owner) { b = best; bsl = slot; }
+}
+
+// Refresh entry points of the kernel: the split forms in the instance that
+// keeps split SM records, the plain ones otherwise.
+template <bool EXT, bool NOC, bool SPL>
+__device__ __forceinline__ void r_sm(const Pt &P, uint32_t s, uint32_t t, uint32_t H, int lane) {
+  if constexpr (SPL) split_refresh_sm(P, s, t, H, lane); else refresh_sm<EXT, NOC>(P, s, t, H, lane);
+}
+template <bool EXT, bool NOC, bool SPL>
+__device__ __forceinline__ void r_sm_owner(const Pt &P, uint32_t s, uint32_t t, uint32_t H, int lane, uint64_t &b,
+                                           uint32_t &bsl) {
+  if constexpr (SPL) split_refresh_sm_owner(P, s, t, H, lane, b, bsl); else refresh_sm_owner<EXT, NOC>(P, s, t, H, lane, b, bsl);
+}
+template <bool EXT, bool NOC, bool SPL>
+__device__ __forceinline__ void r_rescan(const Pt &P, uint32_t s, uint32_t t, uint32_t H) {
+  if constexpr (SPL) split_rescan_sm_lane(P, s, t, H); else rescan_sm_lane<EXT, NOC>(P, s, t, H);
+}
+template <bool SPL>
+__device__ __forceinline__ uint64_t r_lane_best(const Pt &P, int lane, uint32_t H, uint32_t &slot) {
+  if constexpr (SPL) return split_lane_best(P, lane, H, slot); else return lane_best(P, lane, slot);
+}
+template <bool SPL>
+__device__ __forceinline__ void r_owner(const Pt &P, uint32_t owner, int lane, uint32_t H, uint64_t &b, uint32_t &bsl) {
+  if constexpr (SPL) split_refresh_owner(P, owner, lane, H, b, bsl); else refresh_owner(P, owner, lane, b, bsl);
+}
+// SM s's record must be rescanned once H passes its least HBM key (whole records only).
+template <bool SPL>
+__device__ __forceinline__ bool r_stale(const Pt &P, uint32_t s, uint32_t H) {
+  if constexpr (SPL) {
+    const uint2 c = *reinterpret_cast<const uint2 *>(P.smrec(s) + 2);
+    return c.y < H && (c.x >> 16) == 0xFFFFu;
+  } else {
+    return P.smrec(s)[3] < H;
+  }
+}
+
 // Slot i takes node v as its head (v == NONE: stream exhausted); adj_cnt /
 // adj_rdy are releases the caller applied directly.  Every lane writes the
 // same values.
@@ -672,7 +868,7 @@ struct Clock {
 
 // Retire finished CTAs and launch as many CTAs as fit at cycle t (Section 5.1
 // TB scheduler; kernel-boundary gate).  Returns false on step-limit.
-template <bool EXT, bool NOC>
+template <bool EXT, bool NOC, bool SPL>
 __device__ bool launch_ctas(const DevGraph &g, Pt &P, Clock &C, int32_t *cta_sm_row, int lane, uint64_t &b,
                             uint32_t &bsl) {
   const uint32_t t = C.t;
@@ -730,8 +926,8 @@ __device__ bool launch_ctas(const DevGraph &g, Pt &P, Clock &C, int32_t *cta_sm_
     }
     __syncwarp();
     const uint32_t s = div16(freeslot, P.mCps);
-    refresh_sm<EXT, NOC>(P, s, t, C.H, lane);
-    refresh_owner(P, s & 31u, lane, b, bsl);
+    r_sm<EXT, NOC, SPL>(P, s, t, C.H, lane);
+    r_owner<SPL>(P, s & 31u, lane, C.H, b, bsl);
     C.next_cta++;
   }
 }
@@ -820,12 +1016,13 @@ __device__ __forceinline__ void put_constants(uint32_t *sp, const int32_t *prm, 
 
 // EXT: the instances that also run the per-subpartition issue policies and the L2
 // model; NOC: and the NoC of DSMEM nodes, apart because its code costs the others
-// 2%.  The host launches the plainest one that the rows and the graph need.  A
+// 2%; SPL: the plain instance with split SM records, for graphs without edges between
+// CTAs on rows of fewer than SPLIT_SLOTS slots per SM.  The host launches the plainest one that the rows and the graph need.  A
 // warp's registers come from one SM sub-partition's 16K-register file, allocated 8
 // per thread at a time: 4 warps fit per sub-partition up to 128 registers, 3 up to
 // 168, 2 above.  The plain instance is held to 128 (16 warps per SM), the extended
 // ones to 168 (12 warps per SM).
-template <bool EXT, bool NOC>
+template <bool EXT, bool NOC, bool SPL>
 __global__ void __launch_bounds__(MAX_WPB * 32, EXT ? 3 : 4)
 k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point, uint32_t n_points, uint32_t flags,
            int32_t *d_start, int32_t *d_finish, int32_t *d_makespan, int32_t *d_status, uint64_t *d_digest,
@@ -868,7 +1065,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
     const bool l2on = EXT && status == GTS_OK && prm[GTS_P_L2_BYTES] != 0;
     if (status == GTS_OK) {
       if (!make_layout(prm, CG, P.W, g.class_mask, P.L) || P.L.words > budget_words ||
-          (!EXT && (P.L.nsub || prm[GTS_P_L2_BYTES] != 0)) || (!NOC && P.L.cap_noc))
+          (!EXT && (P.L.nsub || prm[GTS_P_L2_BYTES] != 0)) || (!NOC && P.L.cap_noc) || (SPL && P.L.per >= SPLIT_SLOTS))
         status = GTS_ERR_UNSUPPORTED;
     }
     if (status != GTS_OK) {
@@ -913,7 +1110,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
     }
     for (uint32_t s = lane; s < P.L.NS; s += 32) {
       uint32_t *o = P.smrec(s);
-      o[0] = NONE; o[1] = INF; o[2] = 0u; o[3] = INF;
+      o[0] = NONE; o[1] = INF; o[2] = SPL ? SPLIT_NONE : 0u; o[3] = INF;
     }
     for (uint32_t j = lane; j < P.L.Scta; j += 32) P.cta(j)[C_ID] = NONE;
     for (uint32_t k = lane; k < P.L.NS * P.L.SC; k += 32) sp[P.L.o_sv + k] = 0u;
@@ -951,7 +1148,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
     const uint64_t l2_cap = l2on ? (uint64_t)prm[GTS_P_L2_BYTES] : 0ull;
     uint64_t b = INF64;  // this lane's best (effective cycle << 32 | id) over its SMs
     uint32_t bsl = 0;    // ... and its slot
-    if (!launch_ctas<EXT, NOC>(g, P, C, cta_sm_row, lane, b, bsl)) status = GTS_ERR_STEP_LIMIT;
+    if (!launch_ctas<EXT, NOC, SPL>(g, P, C, cta_sm_row, lane, b, bsl)) status = GTS_ERR_STEP_LIMIT;
 
     while (status == GTS_OK && issued < nG) {
       // ---- next event: minimum of (effective cycle, node id) over all heads
@@ -964,7 +1161,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
         if (++C.steps > C.limit) { status = GTS_ERR_STEP_LIMIT; break; }
         C.t = tn;
         if (C.next_ret <= C.t) {  // a CTA retires first: launch, then choose again
-          if (!launch_ctas<EXT, NOC>(g, P, C, cta_sm_row, lane, b, bsl)) { status = GTS_ERR_STEP_LIMIT; break; }
+          if (!launch_ctas<EXT, NOC, SPL>(g, P, C, cta_sm_row, lane, b, bsl)) { status = GTS_ERR_STEP_LIMIT; break; }
           continue;
         }
         // otherwise the minimum just found is the first issue at the new cycle
@@ -1088,11 +1285,11 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
         const bool to_next = mine && ew.x == nx;  // the stream's next node becomes the head right below
         bool to_head = false, cross = false;
         const uint32_t wc = ew.y >> 8;
-        uint32_t tcs = (mine && !to_next && wc == myc) ? cs : NONE;
+        uint32_t tcs = mine && !to_next && (SPL || wc == myc) ? cs : NONE;
         // successors in other CTAs: where the CTAs fit at once, each sits in the slot of its rank; else find each
         // one's slot, all lanes searching together (searching for all of them took 8% of the random DAGs' time
         // and of the fused attention's)
-        bool away = g.cross_cta && mine && !to_next && wc != myc;
+        bool away = !SPL && g.cross_cta && mine && !to_next && wc != myc;
         if (away) {
           const uint32_t rank = wc - P.c0;
           if (rank < P.L.Scta && P.cta(rank)[C_ID] == wc) {
@@ -1100,7 +1297,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
             away = false;
           }
         }
-        uint32_t xm = __ballot_sync(FULL, away);
+        uint32_t xm = SPL ? 0u : __ballot_sync(FULL, away);
         while (xm) {
           const int j = __ffs(xm) - 1;
           xm &= xm - 1;
@@ -1123,14 +1320,14 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
               atomicMax(&ts[F_RDY], rel);
               const uint32_t left = (atomicSub(&ts[F_META], 256u) >> 8) - 1u;
               to_head = true;
-              cross = tcs != cs && left == 0u;  // a head that waits for more predecessors keeps its key: none
+              cross = !SPL && tcs != cs && left == 0u;  // a head that waits for more predecessors keeps its key: none
               if (EXT && cross) xs = div16(tcs, P.mCps);
             }
           }
         }
         adj_cnt += __reduce_add_sync(FULL, to_next ? 1u : 0u);
         adj_rdy = max(adj_rdy, __reduce_max_sync(FULL, to_next ? rel : 0u));
-        cross_touch |= __any_sync(FULL, cross);
+        if (!SPL) cross_touch |= __any_sync(FULL, cross);
         uint32_t todo = __ballot_sync(FULL, mine && !to_next && !to_head);
         while (todo) {
           const int j = __ffs(todo) - 1;
@@ -1151,7 +1348,7 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
       __syncwarp();
       // ---- refresh keys and summaries the issue may have changed
       if (EXT && cross_touch && deg <= 32u) {  // releases reached heads of other CTAs: their SMs and this one
-        refresh_sm<EXT, NOC>(P, sm, t, C.H, lane);
+        r_sm<EXT, NOC, SPL>(P, sm, t, C.H, lane);
         bool own = (uint32_t)lane == (sm & 31u);
         uint32_t xm = __ballot_sync(FULL, xs != NONE && xs != sm);
         uint32_t done = sm;
@@ -1161,84 +1358,97 @@ k_simulate(DevGraph g, const int32_t *__restrict__ params, uint32_t first_point,
           const uint32_t s2 = __shfl_sync(FULL, xs, j);
           if (s2 == done) continue;
           done = s2;
-          refresh_sm<EXT, NOC>(P, s2, t, C.H, lane);
+          r_sm<EXT, NOC, SPL>(P, s2, t, C.H, lane);
           own |= (uint32_t)lane == (s2 & 31u);
         }
         if (C.H != prevH) {  // and the SMs whose HBM heads the new horizon overtakes
           for (uint32_t s = lane; s < P.L.NS; s += 32) {
-            if (P.smrec(s)[3] < C.H) {
-              rescan_sm_lane<EXT, NOC>(P, s, t, C.H);
+            if (r_stale<SPL>(P, s, C.H)) {
+              r_rescan<EXT, NOC, SPL>(P, s, t, C.H);
               own = true;
             }
           }
         }
         if (NOC && noc_touch) {  // the group's other SMs may hold DSMEM heads keyed on that server
           const uint32_t g0 = div16(sm, P.mCsms) * P.L.csms, g1 = min(g0 + P.L.csms, P.L.NS);
-          for (uint32_t s = g0 + lane; s < g1; s += 32) rescan_sm_lane<EXT, NOC>(P, s, t, C.H);
+          for (uint32_t s = g0 + lane; s < g1; s += 32) r_rescan<EXT, NOC, SPL>(P, s, t, C.H);
           __syncwarp();
           for (uint32_t s = g0; s < g1; s++) own |= (s & 31u) == (uint32_t)lane;
         }
         __syncwarp();
-        if (own) b = lane_best(P, lane, bsl);
-      } else if (cross_touch) {  // a node with many successors: recompute everything
-        for (uint32_t s = lane; s < P.L.NS; s += 32) rescan_sm_lane<EXT, NOC>(P, s, t, C.H);
+        if (own) b = r_lane_best<SPL>(P, lane, C.H, bsl);
+      } else if (!SPL && cross_touch) {  // a head of another CTA is ready (extended: by a node of many successors): all SMs
+        for (uint32_t s = lane; s < P.L.NS; s += 32) r_rescan<EXT, NOC, SPL>(P, s, t, C.H);
         __syncwarp();
-        b = lane_best(P, lane, bsl);
-      } else if ((C.H == prevH || P.L.NS == 1u) && P.L.per <= 16u && P.L.NS <= 512u && !(EXT && P.L.nsub)) {
+        b = r_lane_best<SPL>(P, lane, C.H, bsl);
+      } else if ((C.H == prevH || P.L.NS == 1u) && (SPL || P.L.per <= 16u) && P.L.NS <= 512u && !(EXT && P.L.nsub)) {
         // no other SM's record moves
-        refresh_sm_owner<EXT, NOC>(P, sm, t, C.H, lane, b, bsl);
+        r_sm_owner<EXT, NOC, SPL>(P, sm, t, C.H, lane, b, bsl);
         if (NOC && noc_touch) {  // the group's other SMs may hold DSMEM heads keyed on that server
           const uint32_t g0 = div16(sm, P.mCsms) * P.L.csms, g1 = min(g0 + P.L.csms, P.L.NS);
           for (uint32_t s = g0 + lane; s < g1; s += 32)
-            if (s != sm) rescan_sm_lane<EXT, NOC>(P, s, t, C.H);
+            if (s != sm) r_rescan<EXT, NOC, SPL>(P, s, t, C.H);
           __syncwarp();
           bool mine = false;
           for (uint32_t s = g0; s < g1; s++) mine |= s != sm && (s & 31u) == (uint32_t)lane;
-          if (mine) b = lane_best(P, lane, bsl);
+          if (mine) b = r_lane_best<SPL>(P, lane, C.H, bsl);
         }
       } else {
-        refresh_sm<EXT, NOC>(P, sm, t, C.H, lane);
-        if (C.H != prevH && P.L.per >= 8u && !(EXT && P.L.nsub)) {
+        r_sm<EXT, NOC, SPL>(P, sm, t, C.H, lane);
+        if (!SPL && C.H != prevH && P.L.per >= SPLIT_SLOTS && !(EXT && P.L.nsub)) {
           // SMs of many slots: one SM at a time, a slot per lane
           bool own = (uint32_t)lane == (sm & 31u);
           for (uint32_t s0 = 0; s0 < P.L.NS; s0 += 32) {
             const uint32_t s = s0 + lane;
-            uint32_t xm = __ballot_sync(FULL, s < P.L.NS && s != sm && P.smrec(s)[3] < C.H);
+            uint32_t xm = __ballot_sync(FULL, s < P.L.NS && s != sm && r_stale<SPL>(P, s, C.H));
             while (xm) {
               const uint32_t s2 = s0 + __ffs(xm) - 1;
               xm &= xm - 1;
-              refresh_sm<EXT, NOC>(P, s2, t, C.H, lane);
+              r_sm<EXT, NOC, SPL>(P, s2, t, C.H, lane);
               own |= (uint32_t)lane == (s2 & 31u);
             }
           }
-          if (own) b = lane_best(P, lane, bsl);
+          if (own) b = r_lane_best<SPL>(P, lane, C.H, bsl);
+        } else if (SPL && C.H != prevH) {
+          // split records: one pass per lane rescans its whole records that H
+          // overtook and takes its best at the new H from every record it owns
+          uint64_t nb = INF64;
+          uint32_t ns = 0;
+          for (uint32_t s = lane; s < P.L.NS; s += 32) {
+            if (s != sm && r_stale<SPL>(P, s, C.H)) r_rescan<EXT, NOC, SPL>(P, s, t, C.H);
+            uint32_t sl;
+            const uint64_t v = split_sm_best(P, s, C.H, sl);
+            if (v < nb) { nb = v; ns = sl; }
+          }
+          b = nb;
+          bsl = ns;
         } else if (C.H != prevH) {
           // SMs whose HBM heads H overtakes change their effective cycles
           bool any = false;
           for (uint32_t s = lane; s < P.L.NS; s += 32) {
-            if (s != sm && P.smrec(s)[3] < C.H) {
-              rescan_sm_lane<EXT, NOC>(P, s, t, C.H);
+            if (s != sm && r_stale<SPL>(P, s, C.H)) {
+              r_rescan<EXT, NOC, SPL>(P, s, t, C.H);
               any = true;
             }
           }
-          if (any || (uint32_t)lane == (sm & 31u)) b = lane_best(P, lane, bsl);
+          if (any || (uint32_t)lane == (sm & 31u)) b = r_lane_best<SPL>(P, lane, C.H, bsl);
         } else {
-          refresh_owner(P, sm & 31u, lane, b, bsl);
+          r_owner<SPL>(P, sm & 31u, lane, C.H, b, bsl);
         }
         if (NOC && noc_touch) {  // the group's other SMs may hold DSMEM heads keyed on that server
           const uint32_t g0 = div16(sm, P.mCsms) * P.L.csms, g1 = min(g0 + P.L.csms, P.L.NS);
           for (uint32_t s = g0 + lane; s < g1; s += 32)
-            if (s != sm) rescan_sm_lane<EXT, NOC>(P, s, t, C.H);
+            if (s != sm) r_rescan<EXT, NOC, SPL>(P, s, t, C.H);
           __syncwarp();
           bool mine = false;  // this lane owns one of them
           for (uint32_t s = g0; s < g1; s++) mine |= s != sm && (s & 31u) == (uint32_t)lane;
-          if (mine) b = lane_best(P, lane, bsl);
+          if (mine) b = r_lane_best<SPL>(P, lane, C.H, bsl);
         }
       }
       __syncwarp();
       if (rem == 0u) {
         if (cend <= t) {
-          if (!launch_ctas<EXT, NOC>(g, P, C, cta_sm_row, lane, b, bsl)) { status = GTS_ERR_STEP_LIMIT; break; }
+          if (!launch_ctas<EXT, NOC, SPL>(g, P, C, cta_sm_row, lane, b, bsl)) { status = GTS_ERR_STEP_LIMIT; break; }
         } else {
           C.next_ret = min(C.next_ret, cend);
         }
@@ -2067,7 +2277,7 @@ __device__ __forceinline__ uint32_t lane_grant(const DevGraph &g, const LanePt &
 }
 
 // EXT: the instance for tables with rows under the L2 model or an issue policy
-// (96 rows of the L2 study's GEMM 8.3-12 ms, 66.1 in k_simulate<true, false>; 448 rows
+// (96 rows of the L2 study's GEMM 8.3-12 ms, 66.1 in k_simulate<true, false, false>; 448 rows
 // of the policy study 6.0-7.1 for 17.2).
 template <bool EXT>
 __global__ void __launch_bounds__(MAX_WPB * 32, 3)
@@ -2649,6 +2859,7 @@ struct gts_params {
   uint32_t n_points;
   std::vector<uint32_t> words;  // per row: shared words, 0 if the row is invalid or too large
   std::vector<uint8_t> sched;   // per row: asks for a per-subpartition issue policy or the L2 model
+  std::vector<uint8_t> wide;    // per row: SMs of SPLIT_SLOTS or more warp slots
   std::vector<double> cost;     // per row: estimated simulation cost (0 for invalid rows)
   std::vector<float> lcost;      // per row: estimated cost in the lane-parallel instance
   std::vector<uint32_t> lwords;  // per row: shared words in the lane-parallel instance, 0 if it cannot run there
@@ -3066,6 +3277,7 @@ gts_status gts_params_upload(gts_graph *g, const int32_t *d_params, uint32_t n_p
   P->n_points = n_points;
   P->words.assign(n_points, 0u);
   P->sched.assign(n_points, 0u);
+  P->wide.assign(n_points, 0u);
   P->cost.assign(n_points, 0.0);
   P->lwords.assign(n_points, 0u);
   P->ltight.assign(n_points, 0u);
@@ -3078,6 +3290,7 @@ gts_status gts_params_upload(gts_graph *g, const int32_t *d_params, uint32_t n_p
     Layout L;
     if (make_layout(row, g->cta_off[gi + 1] - g->cta_off[gi], g->W, g->dg.class_mask, L)) {
       P->words[p] = L.words;
+      P->wide[p] = L.per >= SPLIT_SLOTS;
       LaneLayout LL;
       if (g->lanes && lane_row_ok(row, g->dg.zero_types) && make_lane_layout(L, true, row[GTS_P_L2_BYTES] ? g->dg.n_tiles : 0u, LL) &&
           lane_pays(L)) {
@@ -3127,6 +3340,7 @@ struct Plan {
   uint32_t words, wpb, smem, blocks, warps;
   bool sched;  // launch the extended instance (issue policies, NoC, L2)
   bool noc;    // ... with the NoC of DSMEM nodes
+  bool split;  // plain instance with split SM records
   bool lanes;  // lane-parallel instance (every valid row can run there)
   bool pad;    // ... with padded slots
   float top;   // cost of the dearest row, 0 when every point starts at once
@@ -3139,6 +3353,7 @@ gts_status plan_launch(const gts_graph *g, const gts_params *P, uint32_t first, 
   pl.top = 0.0f;
   pl.sched = false;
   pl.lanes = true;
+  bool wide = false;
   for (uint32_t p = first; p < first + np; p++) {
     words = std::max(words, P->words[p]);
     lwords = std::max(lwords, P->lwords[p]);
@@ -3146,11 +3361,14 @@ gts_status plan_launch(const gts_graph *g, const gts_params *P, uint32_t first, 
     pl.top = std::max(pl.top, P->lcost[p]);
     pl.lanes = pl.lanes && (P->lwords[p] || !P->words[p]);
     pl.sched = pl.sched || P->sched[p];
+    wide = wide || P->wide[p];
   }
   pl.noc = (g->dg.class_mask & CM_NOC) != 0u;
+  pl.split = !pl.lanes && !pl.sched && !pl.noc && !g->dg.cross_cta && !wide;
   const void *kern = pl.lanes ? (pl.sched ? (const void *)k_simulate_lanes<true> : (const void *)k_simulate_lanes<false>)
-                   : pl.noc ? (const void *)k_simulate<true, true>
-                   : pl.sched ? (const void *)k_simulate<true, false> : (const void *)k_simulate<false, false>;
+                   : pl.noc ? (const void *)k_simulate<true, true, false>
+                   : pl.sched ? (const void *)k_simulate<true, false, false>
+                   : pl.split ? (const void *)k_simulate<false, false, true> : (const void *)k_simulate<false, false, false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   int dev = 0, sms = 0;
@@ -3225,7 +3443,7 @@ int32_t gts_batch_plan(const gts_graph *g, const gts_params *P, uint32_t first_p
   const gts_status st = plan_launch(g, P, first_point, n_points, 0, 0, false, pl);
   if (st != GTS_OK) return st;
   return (pl.lanes ? GTS_PLAN_LANES | (pl.pad ? GTS_PLAN_PADDED : 0) : 0) | (pl.sched || pl.noc ? GTS_PLAN_EXTENDED : 0) |
-         (pl.noc ? GTS_PLAN_NOC : 0);
+         (pl.noc ? GTS_PLAN_NOC : 0) | (pl.split ? GTS_PLAN_SPLIT : 0);
 }
 
 gts_status gts_simulate_batch(gts_graph *g, gts_params *P, uint32_t first_point, uint32_t n_points, uint32_t flags,
@@ -3256,7 +3474,8 @@ gts_status gts_simulate_batch(gts_graph *g, gts_params *P, uint32_t first_point,
       const cudaError_t em = cudaMemsetAsync(d_scratch, 0, GTS_SCRATCH_HEADER_BYTES, s);
       if (em != cudaSuccess) return cuda_fail(em, "simulate: clear the point counter");
     }
-    auto kern = pl.noc ? k_simulate<true, true> : pl.sched ? k_simulate<true, false> : k_simulate<false, false>;
+    auto kern = pl.noc ? k_simulate<true, true, false> : pl.sched ? k_simulate<true, false, false>
+              : pl.split ? k_simulate<false, false, true> : k_simulate<false, false, false>;
     uint64_t *dig = (flags & GTS_WANT_DIGEST) ? d_digest : nullptr;
     int32_t *csm = (flags & GTS_WANT_CTA_SM) ? d_cta_sm : nullptr;
     int64_t *busy = (flags & GTS_WANT_BUSY) ? d_busy : nullptr;

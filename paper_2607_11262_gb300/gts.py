@@ -35,7 +35,7 @@ GTS_WANT_CTA_SM = 4
 GTS_WANT_BUSY = 8
 GTS_SCRATCH_CLEAN = 16
 
-GTS_PLAN_LANES, GTS_PLAN_EXTENDED, GTS_PLAN_NOC, GTS_PLAN_PADDED = 1, 2, 4, 8
+GTS_PLAN_LANES, GTS_PLAN_EXTENDED, GTS_PLAN_NOC, GTS_PLAN_PADDED, GTS_PLAN_SPLIT = 1, 2, 4, 8, 16
 
 GTS_BUSY_CLASSES = 9
 (GTS_BUSY_TENSOR, GTS_BUSY_TMA, GTS_BUSY_LSU, GTS_BUSY_ALU, GTS_BUSY_BAR, GTS_BUSY_HBM, GTS_BUSY_NOC,

@@ -1,12 +1,14 @@
-"""The lean kernel instance with split SM records, which the library launches
-when every row's SMs hold fewer than 8 warp slots, against the oracle and
-against the whole-record instance.
+"""The general kernel's instance with split SM records, which the library launches
+for batches the lane-parallel kernel does not take when every row's SMs hold
+fewer than 8 warp slots, against the oracle and against the whole-record instance.
+Each test states which one it runs.
 
 An SM with exactly one issuable HBM head keeps that head apart in its record
 and takes its effective cycle max(key, H) when the record is read; an SM with
 several HBM heads keeps the whole record and is rescanned when the HBM
 horizon passes its least HBM key.  These graphs are LOAD/STORE heavy with
-several warps per CTA, so both forms occur and the horizon moves often."""
+several warps per CTA, so both forms occur and the horizon moves often; their
+NOPs of no latency keep them out of the lanes."""
 import numpy as np
 import pytest
 
@@ -27,7 +29,8 @@ def _cuda():
     gts.load()
 
 
-HBM_HEAVY = (W.LOAD, W.LOAD, W.STORE, W.MMA, W.EW, W.BAR)
+LANES, SPLIT = 1, 16   # GTS_PLAN_LANES, GTS_PLAN_SPLIT
+HBM_HEAVY = (W.LOAD, W.LOAD, W.LOAD, W.STORE, W.MMA, W.EW, W.BAR, W.NOP)
 
 
 def _rows(rng, k, cps):
@@ -44,9 +47,10 @@ def _rows(rng, k, cps):
 def test_split_instance_against_the_oracle(seed):
     """Rows of 3 warps x 2 CTA slots (6 slots per SM): the split instance."""
     rng = np.random.default_rng(9100 + seed)
-    g = TG.random_graph(rng, 120, W_=3, C=6, p_edge=0.06, types=HBM_HEAVY)
+    g = TG.random_graph(rng, 120, W_=3, C=6, p_edge=0.2, types=HBM_HEAVY, intra_cta=True, cta_major=seed != 2)
     prms = _rows(rng, 12, 2)
     res = H.run_gpu(g, prms)
+    assert res["plan"] == SPLIT
     for q in range(prms.shape[0]):
         H.assert_point_equal(g, prms[q], res, q, oracle_run.simulate(g, prms[q]))
 
@@ -56,12 +60,13 @@ def test_split_and_whole_instances_agree():
     makes the library launch the whole-record instance) give identical
     results to the batch of those rows alone (split instance)."""
     rng = np.random.default_rng(9200)
-    g = TG.random_graph(rng, 150, W_=4, C=6, p_edge=0.05, types=HBM_HEAVY)
+    g = TG.random_graph(rng, 150, W_=4, C=6, p_edge=0.2, types=HBM_HEAVY, intra_cta=True)
     small = _rows(rng, 10, 1)                 # 4 slots per SM
     wide = TG.small_params(rng, num_sms=2, cps=2)   # 8 slots per SM
     mixed = np.concatenate([small, wide[None, :]])
     a = H.run_gpu(g, small)
     b = H.run_gpu(g, mixed)
+    assert (a["plan"], b["plan"]) == (SPLIT, 0)
     n = small.shape[0]
     for k in ("status", "makespan", "digest"):
         assert np.array_equal(a[k], b[k][:n]), k
@@ -74,10 +79,15 @@ def test_split_and_whole_instances_agree():
 
 def test_wsgemm_shape_rows_run_split():
     """The ws GEMM profiling case (3 warps per CTA, 1 CTA per SM) on a few
-    points, spread over the SM-count axis, against the oracle."""
+    points, spread over the SM-count axis, against the oracle: in the lanes, and
+    on 170 CTAs beside a row of 170 SMs, which the lanes cannot take."""
     w = W.workload("wsgemm_small")
     order = np.argsort(w.params[:, W.P_NUM_SMS], kind="stable")
     pts = w.params[order[[0, len(order) // 2, len(order) - 1]]]
-    res = H.run_gpu(w.graph, pts)
-    for q in range(pts.shape[0]):
-        H.assert_point_equal(w.graph, pts[q], res, q, oracle_run.simulate(w.graph, pts[q]))
+    wide = pts[-1:].copy()
+    wide[0, W.P_NUM_SMS] = 170
+    for g, rows, plan in ((w.graph, pts, LANES), (W.ws_gemm(2048, 2048, 256, 170, "ws170"), np.concatenate([pts, wide]), SPLIT)):
+        res = H.run_gpu(g, rows)
+        assert res["plan"] & (LANES | SPLIT) == plan
+        for q in range(rows.shape[0]):
+            H.assert_point_equal(g, rows[q], res, q, oracle_run.simulate(g, rows[q]))

@@ -22,7 +22,7 @@ static std::vector<std::vector<char>> in;
 template <class T> static T *arr(int k) { return reinterpret_cast<T *>(in[k].data()); }
 static DevGraph g;
 static uint32_t h[16];
-static bool lanes, ext, noc, pad;
+static bool lanes, ext, noc, pad, split;
 static int32_t *st, *fi, *mk, *status, *cta_sm;
 static uint64_t *digest;
 static int64_t *busy;
@@ -34,9 +34,10 @@ static void body() {
 #define ARGS g, prm, 0u, np_, f, st, fi, mk, status, digest, cta_sm, busy, scratch, 1u, words, nullptr, 0u
   if (lanes && ext) k_simulate_lanes<true>(ARGS, 0.0f, pad);
   else if (lanes) k_simulate_lanes<false>(ARGS, 0.0f, pad);
-  else if (noc) k_simulate<true, true>(ARGS);
-  else if (ext) k_simulate<true, false>(ARGS);
-  else k_simulate<false, false>(ARGS);
+  else if (noc) k_simulate<true, true, false>(ARGS);
+  else if (ext) k_simulate<true, false, false>(ARGS);
+  else if (split) k_simulate<false, false, true>(ARGS);
+  else k_simulate<false, false, false>(ARGS);
 }
 int main(int, char **argv) {
   FILE *f = fopen(argv[1], "rb");
@@ -50,7 +51,7 @@ int main(int, char **argv) {
   g.cta_cnt = arr<uint32_t>(4); g.cta_kernel = arr<uint32_t>(5); g.node_off = arr<uint32_t>(6); g.cta_off = arr<uint32_t>(7);
   g.W = h[0]; g.G = 1; g.row_nodes = h[1]; g.row_ctas = h[2]; g.cross_cta = h[3]; g.n_tiles = h[4]; g.class_mask = h[5];
   g.zero_types = h[6];
-  np_ = h[7]; lanes = h[8]; ext = h[9]; noc = h[10]; pad = h[11];
+  np_ = h[7]; lanes = h[8]; ext = h[9]; noc = h[10]; pad = h[11]; split = h[13];
   words = 64;
   for (uint32_t p = 0; p < np_; p++) {
     const int32_t *row = arr<int32_t>(9) + p * GTS_NPARAM;
@@ -103,7 +104,7 @@ def build(path, edit=lambda s: s):
     return exe
 
 
-def run(exe, path, g, params, lanes, pad=True, backwards=False):
+def run(exe, path, g, params, lanes, pad=True, backwards=False, split=False):
     """Results of the batch, as tests.gpu_helpers.run_gpu gives them, with ``scratch``, and the sanitizer's report."""
     n, C, Wp = g.n_nodes, g.n_ctas, g.warps_per_cta
     col, cta = g.col.astype(np.int64), g.cta.astype(np.int64)
@@ -130,7 +131,7 @@ def run(exe, path, g, params, lanes, pad=True, backwards=False):
     P = prm.shape[0]
     ext = bool(np.any(prm[:, W.P_ISSUE_POLICY]) or np.any(prm[:, W.P_L2_BYTES]))
     head = np.array([Wp, n, C, int(np.any(cta[src] != cta[col])), n_tiles, mask, zero_types, P, lanes, ext,
-                     bool(mask & 32), pad, backwards, 0, 0, 0], np.uint32)
+                     bool(mask & 32), pad, backwards, split, 0, 0], np.uint32)
     cnt = np.bincount(cta, minlength=C).astype(np.uint32)
     arrays = (rec, rng, succ, first, cnt, g.cta_kernel, g.node_off, g.cta_off, np.zeros(0, np.uint32), prm)
     a, b = os.path.join(path, "in"), os.path.join(path, "out")
