@@ -316,6 +316,16 @@ gts_status gts_params_destroy(gts_params *params);
  * Errors: INVALID_ARG, CUDA. */
 gts_status gts_params_set_order(gts_params *params, uint32_t *d_order, void *stream);
 
+/* Holds the batches of `params` to one of the two kernels, for tests and
+ * measurements; results do not depend on it.  AUTO (the default) takes the one
+ * estimated to take less time for a batch's rows.  LANES is the lane-parallel
+ * kernel where every valid row of a batch can run in it, else the general one.
+ * Ask for gts_scratch_bytes after setting it.  Errors: INVALID_ARG. */
+#define GTS_KERNEL_AUTO    0
+#define GTS_KERNEL_LANES   1
+#define GTS_KERNEL_GENERAL 2
+gts_status gts_params_set_kernel(gts_params *params, uint32_t kernel);
+
 /* Per-point output row lengths (the per-node start and finish cycles and the
  * thread-block placement of Section 5.1): start/finish rows hold
  * gts_row_nodes() entries (the largest graph of the stack), cta_sm rows

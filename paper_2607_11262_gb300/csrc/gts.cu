@@ -64,6 +64,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <new>
@@ -1577,24 +1578,57 @@ __host__ __device__ inline bool lane_row_ok(const int32_t *p, uint32_t zero_type
   return true;
 }
 
-// Rows of one SM leave the lanes nothing to share: the one-SM pipeline study (1,536
-// rows) took 2.2 ms here and 1.97 ms in k_simulate.
-inline bool lane_pays(const Layout &L) { return L.NS >= 2; }
-
-// Estimated cost of a row, from measured points of wsgemm, FlashAttention and
-// decoder tables: cycles per node are those of a round (3,200 + 20 per simulated
-// SM, which the grants and scans grow with) over the SMs that issue in it.  x SMs
-// have work when HBM keeps up with x of them (memory time against the busiest
-// per-SM unit's); x / (1 + x / 30) issue in a round of 32 lanes (measured 7.6 for 8
-// SMs, 5.6 where HBM feeds 6.2 of 108, 21 of 70, 25 of 132).
-__host__ __device__ inline float lane_cost(const float *work, const int32_t *row, float ns, float nodes) {
-  const float mem = work[WK_MEM] / ((float)row[GTS_P_HBM_BPC] * (float)row[GTS_P_CAP_HBM]);
+// How many SMs HBM keeps busy: the busiest per-SM unit's time, all work on one SM, over memory's.
+__host__ __device__ inline float fed_sms(const float *work, const int32_t *row) {
   float sm = work[WK_MEM] / ((float)row[GTS_P_TMA_BPC] * (float)row[GTS_P_CAP_TMA]);
   sm = fmaxf(sm, work[WK_SMEM] / ((float)row[GTS_P_SMEM_BPC] * (float)row[GTS_P_CAP_LSU]));
   sm = fmaxf(sm, work[WK_FMA] / ((float)row[GTS_P_MMA_FMA_PC] * (float)row[GTS_P_CAP_TENSOR]));
   sm = fmaxf(sm, work[WK_EW] / ((float)row[GTS_P_ALU_OPS_PC] * (float)row[GTS_P_CAP_ALU]));
-  const float x = fmaxf(1.0f, fminf(ns, mem > 0.0f ? sm / mem : ns));
+  const float mem = work[WK_MEM] / ((float)row[GTS_P_HBM_BPC] * (float)row[GTS_P_CAP_HBM]);
+  return mem > 0.0f ? sm / mem : 1e9f;
+}
+
+// Estimated cost of a row, from measured points of wsgemm, FlashAttention and
+// decoder tables: cycles per node are those of a round (3,200 + 20 per simulated
+// SM, which the grants and scans grow with) over the SMs that issue in it.  x SMs
+// have work when HBM keeps up with x of them; x / (1 + x / 30) issue in a round of 32
+// lanes (measured 7.6 for 8 SMs, 5.6 where HBM feeds 6.2 of 108, 21 of 70, 25 of 132).
+__host__ __device__ inline float lane_cost(float fed, float ns, float nodes) {
+  const float x = fmaxf(1.0f, fminf(ns, fed));
   return nodes * (3200.0f + 20.0f * ns) * (1.0f + x / 30.0f) / x;
+}
+
+// Cycles per node of a row in the two kernels, for the choice between them.  A lane
+// walks its SM's slots one after the other, so a step of the lanes grows with the
+// slots per SM, and pays when several SMs issue in it; a step of k_simulate walks
+// them side by side but issues one node, and rescans the SMs whose HBM heads the
+// horizon overtakes.  Fitted to 900 tables on a GB300: ws GEMM and attention graphs,
+// 1 to 132 SMs of 3 to 30 slots, 1 to 3,000 rows, HBM at 32 B/cycle and up, GTO with 1
+// and 4 schedulers, round-robin, the L2 model.  Against the better kernel of each table
+// the choice loses 1.0% on the mean (0.4% under a policy); against k_simulate 18% at
+// most (66 SMs of 24 slots, HBM at 32 B/cycle) and 7% under a policy (GTO, 3 SMs of 30
+// slots).  ms in k_simulate and in the lanes, ws GEMM 2048x2048x512
+// on 3,000 rows: one SM, 3 / 30 slots 18.7 / 20.9 and 21.1 / 53.5; 2 SMs 19.4 / 21.0
+// and 13.0 / 29.4; 4 SMs 19.6 / 21.2 and 7.8 / 16.9; 4 SMs with HBM at 32 B/cycle
+// 19.0 / 22.6 and 20.8 / 51.6; 132 SMs 22.0 / 23.3 and 4.0 / 8.3.  Under round-robin,
+// 2048x1024x512, 14 SMs x 30 slots, 300 rows: HBM at 64 B/cycle 11.4 and 17.9, 505 and
+// more 12.0 and 13.0; 3 slots x 132 SMs, 64 rows 8.6 and 3.7.
+struct RowCycles {
+  float lanes, general;
+};
+inline RowCycles row_cycles(float q, const int32_t *row, const Layout &L) {  // q: fed_sms
+  const float ns = (float)L.NS, per = (float)L.per;
+  const float slots = std::min(ns * per, 2600.0f);  // rescans: one lane's SMs overlap with another's
+  if (row[GTS_P_ISSUE_POLICY] != GTS_POLICY_LOWEST_ID) {
+    // HBM-bound, nearly every grant passes waiting picks, and their SMs are refreshed before the next
+    const float x = q >= 0.85f * ns ? ns : std::max(1.0f, std::min(ns, 0.21f * q * std::sqrt(std::sqrt(q))));
+    return {(2720.0f + 255.0f * per + 12.0f * ns) * (1.0f + x / 6.9f) / x,
+            4170.0f + 16.0f * per + 280.0f * (float)L.nsub + 4.4f * std::min(1.0f, 5.1f / q) * slots};
+  }
+  const float x = std::max(1.0f, std::min(ns, 1.45f * std::sqrt(q)));
+  const bool l2 = row[GTS_P_L2_BYTES] != 0;
+  return {((l2 ? 3590.0f : 2150.0f) + 140.0f * per + 11.5f * ns) * (1.0f + x / 10.0f) / x,
+          (l2 ? 4320.0f : 2690.0f) + 4.0f * per + 4.3f * std::min(1.0f, 10.5f / q) * slots};
 }
 
 // Cost classes of a batch whose dearest row costs `top`: its points are handed out
@@ -1628,7 +1662,7 @@ __device__ __noinline__ uint32_t lane_next_point(const DevGraph *g, const int32_
       if (gi >= 0 && (uint32_t)gi < g->G && cps >= 1) {
         const float ctas = (float)(g->cta_off[gi + 1] - g->cta_off[gi]);
         const float ns = fminf((float)row[GTS_P_NUM_SMS], ceilf(ctas / (float)cps));
-        cls = lane_class(lane_cost(g->work, row, ns, (float)(g->node_off[gi + 1] - g->node_off[gi])), top);
+        cls = lane_class(lane_cost(fed_sms(g->work, row), ns, (float)(g->node_off[gi + 1] - g->node_off[gi])), top);
       }
       if (cls != c) continue;
     }
@@ -2864,6 +2898,8 @@ struct gts_params {
   std::vector<float> lcost;      // per row: estimated cost in the lane-parallel instance
   std::vector<uint32_t> lwords;  // per row: shared words in the lane-parallel instance, 0 if it cannot run there
   std::vector<uint32_t> ltight;  // ... without padded slots
+  std::vector<RowCycles> cycles;  // per row: estimated cycles in either kernel, for the choice (0 if it cannot run in lanes)
+  uint32_t kernel = GTS_KERNEL_AUTO;
   const uint32_t *d_order = nullptr;  // processing order (gts_params_set_order), borrowed
 };
 
@@ -3282,6 +3318,7 @@ gts_status gts_params_upload(gts_graph *g, const int32_t *d_params, uint32_t n_p
   P->lwords.assign(n_points, 0u);
   P->ltight.assign(n_points, 0u);
   P->lcost.assign(n_points, 0.0f);
+  P->cycles.assign(n_points, RowCycles{0.0f, 0.0f});
   for (uint32_t p = 0; p < n_points; p++) {
     const int32_t *row = h.data() + (size_t)p * GTS_NPARAM;
     if (check_row(row, g->G, g->dg.class_mask) != GTS_OK) continue;
@@ -3292,12 +3329,16 @@ gts_status gts_params_upload(gts_graph *g, const int32_t *d_params, uint32_t n_p
       P->words[p] = L.words;
       P->wide[p] = L.per >= SPLIT_SLOTS;
       LaneLayout LL;
-      if (g->lanes && lane_row_ok(row, g->dg.zero_types) && make_lane_layout(L, true, row[GTS_P_L2_BYTES] ? g->dg.n_tiles : 0u, LL) &&
-          lane_pays(L)) {
+      if (g->lanes && lane_row_ok(row, g->dg.zero_types) && make_lane_layout(L, true, row[GTS_P_L2_BYTES] ? g->dg.n_tiles : 0u, LL)) {
         P->lwords[p] = LL.words;
         make_lane_layout(L, false, row[GTS_P_L2_BYTES] ? g->dg.n_tiles : 0u, LL);
         P->ltight[p] = LL.words;
-        P->lcost[p] = lane_cost(g->dg.work, row, (float)L.NS, (float)(g->node_off[gi + 1] - g->node_off[gi]));
+        const float nodes = (float)(g->node_off[gi + 1] - g->node_off[gi]);
+        const float fed = fed_sms(g->dg.work, row);
+        P->lcost[p] = lane_cost(fed, (float)L.NS, nodes);
+        P->cycles[p] = row_cycles(fed, row, L);
+        P->cycles[p].lanes *= nodes;
+        P->cycles[p].general *= nodes;
       }
       // per issue the work grows slowly with the simulated SMs; the extended model costs about 3.5x
       P->cost[p] = (double)(g->node_off[gi + 1] - g->node_off[gi]) * (743.0 + L.NS) * (P->sched[p] ? 3.5 : 1.0);
@@ -3322,6 +3363,13 @@ gts_status gts_params_set_order(gts_params *P, uint32_t *d_order, void *stream) 
   return GTS_OK;
 }
 
+gts_status gts_params_set_kernel(gts_params *P, uint32_t kernel) {
+  clear_error();
+  if (!P || kernel > GTS_KERNEL_GENERAL) return fail(GTS_ERR_INVALID_ARG, "null params or unknown kernel");
+  P->kernel = kernel;
+  return GTS_OK;
+}
+
 gts_status gts_params_destroy(gts_params *p) {
   delete p;
   return GTS_OK;
@@ -3341,14 +3389,31 @@ struct Plan {
   bool sched;  // launch the extended instance (issue policies, NoC, L2)
   bool noc;    // ... with the NoC of DSMEM nodes
   bool split;  // plain instance with split SM records
-  bool lanes;  // lane-parallel instance (every valid row can run there)
+  bool lanes;  // lane-parallel instance (every valid row can run there, and it is estimated to take less time)
   bool pad;    // ... with padded slots
   float top;   // cost of the dearest row, 0 when every point starts at once
 };
 
-gts_status plan_launch(const gts_graph *g, const gts_params *P, uint32_t first, uint32_t np, uint32_t flags,
+// The kernel for a batch: the lanes when every valid row can run there and they are
+// estimated to take less time -- the dearest row's, or all rows' over the warps that
+// share the GPU, of which 7.5 per SM in the lanes and 9 in k_simulate make headway at
+// a time.  One row that cannot run in lanes sends its batch to k_simulate.
+bool lanes_chosen(const gts_params *P, uint32_t first, uint32_t np, uint32_t words, uint32_t lwords, int sms, uint32_t kernel) {
+  if (kernel != GTS_KERNEL_AUTO) return kernel == GTS_KERNEL_LANES;
+  double l = 0.0, gen = 0.0, lmax = 0.0, gmax = 0.0;
+  for (uint32_t p = first; p < first + np; p++) {
+    const RowCycles c = P->cycles[p];
+    l += c.lanes;
+    gen += c.general;
+    lmax = std::max(lmax, (double)c.lanes);
+    gmax = std::max(gmax, (double)c.general);
+  }
+  auto warps = [&](uint32_t w, double most) { return sms * std::min(most, (double)(MAX_SMEM_BYTES / (w * 4))); };
+  return std::max(lmax, l / warps(lwords, 7.5)) <= std::max(gmax, gen / warps(words, 9.0));
+}
+
+gts_status plan_launch(const gts_graph *g, const gts_params *P, uint32_t first, uint32_t np, uint32_t kernel,
                        size_t scratch_bytes, bool limit_by_scratch, Plan &pl) {
-  (void)flags;
   uint32_t words = 64, lwords = 64, ltight = 64;
   pl.top = 0.0f;
   pl.sched = false;
@@ -3363,17 +3428,19 @@ gts_status plan_launch(const gts_graph *g, const gts_params *P, uint32_t first, 
     pl.sched = pl.sched || P->sched[p];
     wide = wide || P->wide[p];
   }
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return cuda_fail(e, "simulate: device attributes");
+  pl.lanes = pl.lanes && lanes_chosen(P, first, np, words, lwords, sms, kernel);
   pl.noc = (g->dg.class_mask & CM_NOC) != 0u;
   pl.split = !pl.lanes && !pl.sched && !pl.noc && !g->dg.cross_cta && !wide;
   const void *kern = pl.lanes ? (pl.sched ? (const void *)k_simulate_lanes<true> : (const void *)k_simulate_lanes<false>)
                    : pl.noc ? (const void *)k_simulate<true, true, false>
                    : pl.sched ? (const void *)k_simulate<true, false, false>
                    : pl.split ? (const void *)k_simulate<false, false, true> : (const void *)k_simulate<false, false, false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM_BYTES);
+  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MAX_SMEM_BYTES);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-  int dev = 0, sms = 0;
-  if (e == cudaSuccess) e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return cuda_fail(e, "simulate: kernel attributes");
   // warps per block: whichever keeps the most design points resident per SM
   auto resident = [&](uint32_t bytes, uint32_t &best_w, uint32_t &best_wpb) {
@@ -3429,9 +3496,22 @@ gts_status plan_launch(const gts_graph *g, const gts_params *P, uint32_t first, 
 
 size_t gts_scratch_bytes(const gts_graph *g, const gts_params *P, uint32_t flags) {
   if (!g || !P) return 0;
-  Plan pl;
-  if (plan_launch(g, P, 0, P->n_points, flags, 0, false, pl) != GTS_OK) return 0;
-  return GTS_SCRATCH_HEADER_BYTES + (size_t)pl.warps * scratch_row_bytes(g);
+  (void)flags;
+  // a part of the table may run in the other kernel, which may have more warps: where the rows differ in which suits them
+  // better, the scratch is sized for both
+  bool l = false, gen = false;
+  for (const RowCycles &c : P->cycles) {
+    l = l || c.lanes < c.general;
+    gen = gen || c.lanes > c.general;
+  }
+  uint32_t warps = 0;
+  for (uint32_t k : {P->kernel, (uint32_t)GTS_KERNEL_LANES, (uint32_t)GTS_KERNEL_GENERAL}) {
+    Plan pl;
+    if (plan_launch(g, P, 0, P->n_points, k, 0, false, pl) != GTS_OK) return 0;
+    warps = std::max(warps, pl.warps);
+    if (P->kernel != GTS_KERNEL_AUTO || !l || !gen) break;
+  }
+  return GTS_SCRATCH_HEADER_BYTES + (size_t)warps * scratch_row_bytes(g);
 }
 
 int32_t gts_batch_plan(const gts_graph *g, const gts_params *P, uint32_t first_point, uint32_t n_points) {
@@ -3440,7 +3520,7 @@ int32_t gts_batch_plan(const gts_graph *g, const gts_params *P, uint32_t first_p
   if ((uint64_t)first_point + n_points > P->n_points) return fail(GTS_ERR_INVALID_ARG, "point range outside the table");
   if (!n_points) return 0;
   Plan pl;
-  const gts_status st = plan_launch(g, P, first_point, n_points, 0, 0, false, pl);
+  const gts_status st = plan_launch(g, P, first_point, n_points, P->kernel, 0, false, pl);
   if (st != GTS_OK) return st;
   return (pl.lanes ? GTS_PLAN_LANES | (pl.pad ? GTS_PLAN_PADDED : 0) : 0) | (pl.sched || pl.noc ? GTS_PLAN_EXTENDED : 0) |
          (pl.noc ? GTS_PLAN_NOC : 0) | (pl.split ? GTS_PLAN_SPLIT : 0);
@@ -3468,7 +3548,7 @@ gts_status gts_simulate_batch(gts_graph *g, gts_params *P, uint32_t first_point,
   cudaStream_t s = (cudaStream_t)stream;
   if (n_points) {
     Plan pl;
-    gts_status st = plan_launch(g, P, first_point, n_points, flags, scratch_bytes, true, pl);
+    gts_status st = plan_launch(g, P, first_point, n_points, P->kernel, scratch_bytes, true, pl);
     if (st != GTS_OK) return st;
     if (P->d_order) {  // the next-point counter
       const cudaError_t em = cudaMemsetAsync(d_scratch, 0, GTS_SCRATCH_HEADER_BYTES, s);

@@ -35,6 +35,7 @@ GTS_WANT_CTA_SM = 4
 GTS_WANT_BUSY = 8
 GTS_SCRATCH_CLEAN = 16
 
+GTS_KERNEL_AUTO, GTS_KERNEL_LANES, GTS_KERNEL_GENERAL = 0, 1, 2
 GTS_PLAN_LANES, GTS_PLAN_EXTENDED, GTS_PLAN_NOC, GTS_PLAN_PADDED, GTS_PLAN_SPLIT = 1, 2, 4, 8, 16
 
 GTS_BUSY_CLASSES = 9
@@ -49,7 +50,7 @@ GTS_STATIC_SCRATCH_BYTES = 32 << 20
 GTS_SCRATCH_HEADER_BYTES = 16
 
 EXPORTS = ("gts_graph_workspace_bytes", "gts_graph_create", "gts_graph_destroy", "gts_template_workspace_bytes",
-           "gts_graph_create_templated", "gts_params_upload", "gts_params_set_order",
+           "gts_graph_create_templated", "gts_params_upload", "gts_params_set_order", "gts_params_set_kernel",
            "gts_params_destroy", "gts_row_nodes", "gts_row_ctas", "gts_scratch_bytes", "gts_batch_plan", "gts_simulate_batch",
            "gts_read_results", "gts_results_destroy", "gts_simulate_batch_noalloc", "gts_last_error")
 
@@ -111,6 +112,8 @@ def load():
     lib.gts_params_destroy.restype = i32
     lib.gts_params_set_order.argtypes = [vp, vp, vp]
     lib.gts_params_set_order.restype = i32
+    lib.gts_params_set_kernel.argtypes = [vp, u32]
+    lib.gts_params_set_kernel.restype = i32
     lib.gts_row_nodes.argtypes = [vp]
     lib.gts_row_nodes.restype = u32
     lib.gts_row_ctas.argtypes = [vp]
@@ -176,6 +179,10 @@ def gts_params_destroy(params):
 
 def gts_params_set_order(params, d_order: int, stream: int = 0):
     _check(load().gts_params_set_order(params, d_order, stream))
+
+
+def gts_params_set_kernel(params, kernel):
+    _check(load().gts_params_set_kernel(params, kernel))
 
 
 def gts_row_nodes(graph):

@@ -42,7 +42,7 @@ def aux_digest(cta_sm, busy):
         return int((int(t1) + int(t2)) & MASK64)
 
 
-def run_gpu(graph, params, flags=None, first_point=0, n_points=None):
+def run_gpu(graph, params, flags=None, first_point=0, n_points=None, kernel=0):
     import torch
 
     from paper_2607_11262_gb300 import gts
@@ -50,6 +50,7 @@ def run_gpu(graph, params, flags=None, first_point=0, n_points=None):
         flags = gts.GTS_FULL_TRACE | gts.GTS_WANT_DIGEST | gts.GTS_WANT_CTA_SM | gts.GTS_WANT_BUSY
     dg = gts.DeviceGraph(graph)
     dp = gts.DeviceParams(dg, params)
+    gts.gts_params_set_kernel(dp.handle, kernel)
     out = gts.simulate(dg, dp, first_point=first_point, n_points=n_points, flags=flags)
     torch.cuda.synchronize()
     res = {"status": out.status.cpu().numpy(), "makespan": out.makespan.cpu().numpy(),

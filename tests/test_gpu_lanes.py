@@ -1,11 +1,11 @@
 """The lane-parallel kernel instance (one simulated SM per lane), which the
-library launches when every valid row has at least two SMs and the graph's ids
-are in CTA order with no edge between CTAs: against the oracle where its tiles
+library can launch when the graph's ids are in CTA order with no edge between
+CTAs and every valid row has up to 160 SMs of up to 32 warp slots: against the oracle where its tiles
 end (SMs per lane round, slots read four at a time, the inline successors,
 servers kept in registers up to four, L2 lists in shared memory), and against
-the general instance, which the same rows run in when the batch also holds a row
-of 33 warp slots on an SM.  Each test states the kernel it means (H.run_gpu gives
-the plan).  Integer results, compared bit for bit."""
+the general instance on the same rows.  The tests hold their batches to the kernel
+they mean and assert that it ran (H.run_gpu gives the plan); which one a batch gets
+by itself has tests of its own.  Integer results, compared bit for bit."""
 import numpy as np
 import pytest
 
@@ -48,7 +48,8 @@ def _row(rng, sms, cps, cap_hbm=1, cap_tma=1, cap_lsu=4):
     return p
 
 
-LANES = 1   # GTS_PLAN_LANES
+LANES = 1             # GTS_PLAN_LANES
+IN_LANES, IN_GENERAL = 1, 2   # GTS_KERNEL_*
 
 
 def _check(g, rows, res, lanes=True):
@@ -64,7 +65,16 @@ def test_sm_counts(sms):
     for mix in range(4):
         g = _graph(rng, 700, 170, 2, mix, kernels=mix == 3)
         rows = np.stack([_row(rng, sms, 1, cap_hbm=c) for c in (1, 1, 3)])
-        _check(g, rows, H.run_gpu(g, rows), lanes=sms <= 160)
+        _check(g, rows, H.run_gpu(g, rows, kernel=IN_LANES), lanes=sms <= 160)
+
+
+@pytest.mark.parametrize("sms", [1, 2, 40])
+def test_rows_of_one_sm(sms):
+    """A row of one SM, alone and beside another."""
+    rng = np.random.default_rng(7050 + sms)
+    g = _graph(rng, 300, 40, 3, 0)
+    rows = np.stack([_row(rng, 1, 2, cap_hbm=2), _row(rng, sms, 1)])
+    _check(g, rows, H.run_gpu(g, rows, kernel=IN_LANES))
 
 
 @pytest.mark.parametrize("warps,cps", [(1, 1), (3, 1), (4, 1), (5, 1), (3, 3), (8, 4), (11, 3)])
@@ -73,7 +83,7 @@ def test_slots_per_sm(warps, cps):
     rng = np.random.default_rng(7100 + warps * cps)
     g = _graph(rng, 300, 20, warps, 0, kernels=True)
     rows = np.stack([_row(rng, s, cps) for s in (2, 3, 5)])
-    _check(g, rows, H.run_gpu(g, rows), lanes=warps * cps <= 32)
+    _check(g, rows, H.run_gpu(g, rows, kernel=IN_LANES), lanes=warps * cps <= 32)
 
 
 @pytest.mark.parametrize("caps", [(1, 1, 1), (2, 2, 2), (4, 4, 4), (1, 5, 5), (32, 32, 32)])
@@ -82,7 +92,7 @@ def test_server_counts(caps):
     for mix in (0, 3):
         g = _graph(rng, 260, 30, 4, mix)
         rows = np.stack([_row(rng, int(rng.choice([2, 7, 33])), int(rng.integers(1, 3)), *caps) for _ in range(6)])
-        _check(g, rows, H.run_gpu(g, rows))
+        _check(g, rows, H.run_gpu(g, rows, kernel=IN_LANES))
 
 
 @pytest.mark.parametrize("fan", [1, 2, 3, 6, 7, 8, 40])
@@ -97,7 +107,7 @@ def test_successor_counts(fan):
                 warps * ctas, [c for c in range(ctas) for _ in range(n)], 3,
                 work=[int(x) for x in rng.integers(1, 9, n * ctas)])
     rows = np.stack([_row(rng, s, c) for s, c in ((2, 1), (3, 2), (8, 1))])
-    _check(g, rows, H.run_gpu(g, rows))
+    _check(g, rows, H.run_gpu(g, rows, kernel=IN_LANES))
 
 
 @pytest.mark.parametrize("mix", range(4))
@@ -107,20 +117,12 @@ def test_nodes_without_work(mix):
     g = _graph(rng, 300, 40, 3, mix, kernels=mix == 1)
     g.work[rng.random(g.n_nodes) < 0.4] = 0
     rows = np.stack([_row(rng, s, c, h) for s, c, h in ((2, 1, 1), (5, 2, 2), (33, 1, 1), (40, 1, 3))])
-    _check(g, rows, H.run_gpu(g, rows))
-
-
-def _beside_33_slots(rng, g, rows):
-    """The rows of a batch that runs in the general kernel because of one more row."""
-    wide = _row(rng, 2, -(-33 // g.warps_per_cta))
-    res = H.run_gpu(g, np.concatenate([rows, wide[None, :]]))
-    assert not res["plan"] & LANES
-    return res
+    _check(g, rows, H.run_gpu(g, rows, kernel=IN_LANES))
 
 
 @pytest.mark.parametrize("seed", range(6))
 def test_agrees_with_the_general_instance(seed):
-    """Rows over all forms the rule takes, alone and beside a row of 33 slots per SM."""
+    """Rows over all forms the rule takes, in either kernel."""
     rng = np.random.default_rng(7400 + seed)
     g = _graph(rng, 400, int(rng.integers(20, 60)), int(rng.integers(1, 7)), seed % 4, kernels=seed % 2 == 1,
                max_work=[2, 6, 60][seed % 3], p_issue=[0.0, 0.3, 0.9][seed % 3])
@@ -130,9 +132,10 @@ def test_agrees_with_the_general_instance(seed):
                      for _ in range(24)])
     rows[7, W.P_TMA_BPC] = 0                    # refused
     rows[11, W.P_DRAM_LAT] = 2**31 - 40         # overflows
-    lanes = H.run_gpu(g, rows)
+    lanes = H.run_gpu(g, rows, kernel=IN_LANES)
     assert lanes["plan"] & LANES
-    both = _beside_33_slots(rng, g, rows)
+    both = H.run_gpu(g, rows, kernel=IN_GENERAL)
+    assert not both["plan"] & LANES
     n = rows.shape[0]
     for k in ("status", "makespan"):
         assert np.array_equal(lanes[k], both[k][:n]), k
@@ -151,7 +154,7 @@ def test_empty_ctas_and_gates():
     g.cta_kernel = np.array([0] * 5 + [1] * 6 + [2] * 10, np.uint32)
     g.cta_off = np.array([0, 21], np.uint32)
     rows = np.stack([_row(rng, s, c) for s, c in ((2, 1), (3, 2), (30, 1))])
-    _check(g, rows, H.run_gpu(g, rows))
+    _check(g, rows, H.run_gpu(g, rows, kernel=IN_LANES))
 
 
 def test_points_taken_by_cost_class():
@@ -162,6 +165,7 @@ def test_points_taken_by_cost_class():
     w = W.workload("wsgemm_small", points=120)
     dg = gts.DeviceGraph(w.graph)
     dp = gts.DeviceParams(dg, w.params)
+    gts.gts_params_set_kernel(dp.handle, IN_LANES)
     row = (dg.row_nodes + 1) // 2 * 16
     assert gts.gts_batch_plan(dg.handle, dp.handle, 0, 120) & LANES
     few = torch.zeros(gts.GTS_SCRATCH_HEADER_BYTES + 7 * row, dtype=torch.uint8, device="cuda")
@@ -185,6 +189,7 @@ def test_dense_slots_agree_with_padded_ones(k):
     p[0, W.P_NUM_SMS] = 132
     dg = gts.DeviceGraph(g)
     dp = gts.DeviceParams(dg, p)
+    gts.gts_params_set_kernel(dp.handle, IN_LANES)
     flags = gts.GTS_WANT_DIGEST | gts.GTS_WANT_BUSY
     assert gts.gts_batch_plan(dg.handle, dp.handle, 0, 3000) == LANES
     whole = gts.simulate(dg, dp, flags=flags)
@@ -214,7 +219,7 @@ def test_l2_lists(tiles):
         g.n_tiles = tiles
         rows = [_row(rng, int(rng.choice([2, 5, 40])), int(rng.integers(1, 3)), int(rng.integers(1, 3))) for _ in range(5)]
         rows = np.stack([rows[0]] + [_with_l2(rng, p, [1, 6, 30, 10**6]) for p in rows[1:]])
-        _check(g, rows, H.run_gpu(g, rows))
+        _check(g, rows, H.run_gpu(g, rows, kernel=IN_LANES))
 
 
 @pytest.mark.parametrize("tiles", [28906, 28907])
@@ -228,7 +233,7 @@ def test_l2_list_limit(tiles):
     g.n_tiles = tiles
     rows = np.stack([_with_l2(rng, _row(rng, 2, 1), [1, 30, 200, 10**6]) for _ in range(4)])
     rows[:, W.P_CAP_TENSOR:W.P_CAP_HBM + 1] = 1
-    _check(g, rows, H.run_gpu(g, rows), lanes=tiles == 28906)
+    _check(g, rows, H.run_gpu(g, rows, kernel=IN_LANES), lanes=tiles == 28906)
 
 
 @pytest.mark.parametrize("schedulers", [1, 2, 3, 4, 7, 32])
@@ -248,7 +253,7 @@ def test_issue_policies(policy, schedulers):
                 p[W.P_ISSUE_POLICY], p[W.P_SUBPARTITIONS] = policy, schedulers
             rows.append(_with_l2(rng, p, [8, 40]) if k == 5 else p)
         rows = np.stack(rows)
-        _check(g, rows, H.run_gpu(g, rows))
+        _check(g, rows, H.run_gpu(g, rows, kernel=IN_LANES))
 
 
 @pytest.mark.parametrize("seed", range(4))
@@ -261,9 +266,58 @@ def test_policies_agree_with_the_general_instance(seed):
         p[W.P_ISSUE_POLICY], p[W.P_SUBPARTITIONS] = 1 + k % 2, int(rng.choice([1, 2, 4]))
         rows.append(p)
     rows = np.stack(rows)
-    lanes = H.run_gpu(g, rows)
+    lanes = H.run_gpu(g, rows, kernel=IN_LANES)
     assert lanes["plan"] & LANES
-    both = _beside_33_slots(rng, g, rows)
+    both = H.run_gpu(g, rows, kernel=IN_GENERAL)
+    assert not both["plan"] & LANES
     assert np.all(lanes["status"] == 0)
     for k in ("status", "makespan", "start", "finish", "digest", "cta_sm", "busy"):
         assert np.array_equal(lanes[k], both[k][:rows.shape[0]]), k
+
+
+def _ws_rows(n, sms, cps, hbm=None, policy=0, schedulers=0):
+    p = W.sweep_params(7, n, [W.AX_SMS, W.AX_HBM, W.AX_TMA_LAT, W.AX_MMA_RATE], 1)
+    p[:, W.P_NUM_SMS], p[:, W.P_CTAS_PER_SM] = sms, cps
+    if hbm:
+        p[:, W.P_HBM_BPC] = hbm
+    p[:, W.P_ISSUE_POLICY], p[:, W.P_SUBPARTITIONS] = policy, schedulers
+    return p
+
+
+@pytest.mark.parametrize("rows,lanes", [
+    ((12, 132, 1), True), ((12, 132, 10), True), ((12, 2, 1), True), ((12, 4, 10), True), ((12, 1, 1), False),
+    ((12, 2, 10), False), ((12, 4, 10, 32), False), ((12, 132, 1, 0, W.POLICY_RR, 1), True),
+    ((12, 3, 1, 0, W.POLICY_GTO, 4), True), ((12, 132, 10, 64, W.POLICY_RR, 1), False),
+    ((12, 2, 10, 0, W.POLICY_GTO, 4), False)])
+def test_the_kernel_that_takes_less_time_runs(rows, lanes):
+    """Rows on both sides of the estimate: SMs that a lane walks 30 slots of, few SMs, HBM that feeds one, policies."""
+    g = W.ws_gemm(2048, 1024, 128, 132, "ws")
+    p = _ws_rows(*rows)
+    res = H.run_gpu(g, p)
+    assert bool(res["plan"] & LANES) == lanes
+    other = H.run_gpu(g, p, kernel=IN_GENERAL if lanes else IN_LANES)
+    assert bool(other["plan"] & LANES) != lanes
+    for k in ("status", "makespan", "start", "finish", "digest", "cta_sm", "busy"):
+        assert np.array_equal(res[k], other[k]), k
+
+
+def test_one_row_does_not_decide_for_the_table():
+    """A sweep that starts at one SM runs in the lanes; scratch from the whole table serves any part of it."""
+    import torch
+
+    from paper_2607_11262_gb300 import gts
+    g = W.ws_gemm(2048, 1024, 128, 132, "ws")
+    p = np.concatenate([_ws_rows(40, 1, 1), _ws_rows(400, 132, 1)])
+    dg = gts.DeviceGraph(g)
+    dp = gts.DeviceParams(dg, p)
+    assert gts.gts_batch_plan(dg.handle, dp.handle, 0, 440) & LANES
+    assert not gts.gts_batch_plan(dg.handle, dp.handle, 0, 40) & LANES
+    scratch = gts.alloc_scratch(dg, dp)
+    flags = gts.GTS_WANT_DIGEST | gts.GTS_SCRATCH_CLEAN
+    whole = gts.simulate(dg, dp, flags=flags, scratch=scratch)
+    for lo, n in ((0, 40), (30, 300), (200, 240)):
+        part = gts.simulate(dg, dp, first_point=lo, n_points=n, flags=flags, scratch=scratch)
+        torch.cuda.synchronize()
+        assert torch.equal(whole.digest[lo:lo + n], part.digest) and torch.equal(whole.makespan[lo:lo + n], part.makespan)
+    assert int(whole.status.abs().sum()) == 0
+    assert int(torch.count_nonzero(scratch[gts.GTS_SCRATCH_HEADER_BYTES:])) == 0

@@ -37,17 +37,13 @@ def test_on_the_host(warp, lanes):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("one_sm_row", [False, True])
-def test_on_the_gpu(one_sm_row):
+@pytest.mark.parametrize("kernel", [1, 2])   # GTS_KERNEL_LANES, GTS_KERNEL_GENERAL
+def test_on_the_gpu(kernel):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     g, rows, refs = _batch()
-    batch = rows
-    if one_sm_row:
-        p = TG.unit_params(1, 1)
-        p[W.P_TMA_LAT] = 1
-        batch = np.concatenate([rows, p[None, :]])
-    res = H.run_gpu(g, batch)
+    res = H.run_gpu(g, rows, kernel=kernel)
+    assert res["plan"] & 1 == (kernel == 1)   # GTS_PLAN_LANES
     for q, ref in enumerate(refs):
         H.assert_point_equal(g, rows[q], res, q, ref)
