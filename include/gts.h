@@ -310,8 +310,10 @@ gts_status gts_params_destroy(gts_params *params);
  * simulated SMs), x 3.5 for rows that need the extended model), and makes
  * gts_simulate_batch hand points to its warps in that order, each warp taking
  * the next point when it finishes one (longest processing time first, which
- * keeps the last wave short; the lane-parallel kernel goes through the order
- * once per cost class, dearest first).  Results do not depend on the order.  Without
+ * keeps the last wave short).  The cost is the general kernel's; in a
+ * lane-parallel batch of more points than warps the order holds within classes
+ * of the lanes' own estimate (above 0.55, 0.4 and 0.3 of the dearest row's, and
+ * the rest), which are handed out dearest first.  Results do not depend on the order.  Without
  * one, warp w takes points w, w + warps, ... .  Waits for `stream`.
  * Errors: INVALID_ARG, CUDA. */
 gts_status gts_params_set_order(gts_params *params, uint32_t *d_order, void *stream);

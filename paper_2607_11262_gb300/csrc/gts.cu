@@ -1633,7 +1633,10 @@ inline RowCycles row_cycles(float q, const int32_t *row, const Layout &L) {  // 
 
 // Cost classes of a batch whose dearest row costs `top`: its points are handed out
 // class by class, in the table's order inside a class, so that the dearest do not
-// start last.  One class when every point starts at once (top = 0).
+// start last.  One class when every point starts at once (top = 0).  ms of ws GEMM
+// 4096x4096x2048 on 3,000 rows and 2048x2048x1024 on 1,500 (3 seeds): 58.9 and 4.98;
+// with bounds 0.7, 0.5, 0.35 58.4 and 5.16; 0.5, 0.25, 0.12 59.5 and 5.01; one class
+// 61.8 and 6.21.
 constexpr uint32_t LANE_CLASSES = 4;
 __device__ __forceinline__ uint32_t lane_class(float cost, float top) {
   return cost > 0.55f * top ? 0u : cost > 0.4f * top ? 1u : cost > 0.3f * top ? 2u : 3u;
@@ -2249,7 +2252,9 @@ __device__ __forceinline__ uint32_t lane_grant(const DevGraph &g, const LanePt &
         X.loads += tile ? ti & 1u : 0u;
       }
     }
-    if (EXT && X.cap) __syncwarp();  // the list is in shared memory and another lane may win the next turn
+    // the L2 list is in shared memory and another lane may win the next turn (with rows of an L2 only, the policies took
+    // 0.8% and the L2 study 1.8% longer)
+    if (EXT) __syncwarp();
     ho = __reduce_max_sync(FULL, win ? ho : 0u);
     const bool takes = !EXT || ho != NONE;
     if (takes && (uint64_t)t + ho > 0x7FFFFFFFull) return NONE;
@@ -2310,9 +2315,11 @@ __device__ __forceinline__ uint32_t lane_grant(const DevGraph &g, const LanePt &
   return n_granted;
 }
 
-// EXT: the instance for tables with rows under the L2 model or an issue policy
-// (96 rows of the L2 study's GEMM 8.3-12 ms, 66.1 in k_simulate<true, false, false>; 448 rows
-// of the policy study 6.0-7.1 for 17.2).
+// EXT: the instance for tables with rows under the L2 model or an issue policy (96 rows
+// of the L2 study's GEMM 7.9-9.3 ms, 66.1 in k_simulate<true, false, false>; 448 rows of
+// the policy study 6.5-7.3 for 17.2).  All rows of such a table run in it: one GTO row
+// among 3,000 lowest-id ones takes the ws GEMM table from 50.6 to 90.1 ms, one among
+// 1,500 rows of the smaller GEMM from 4.90 to 8.67.
 template <bool EXT>
 __global__ void __launch_bounds__(MAX_WPB * 32, 3)
 k_simulate_lanes(const __grid_constant__ DevGraph g, const int32_t *__restrict__ params, uint32_t first_point, uint32_t n_points, uint32_t flags,

@@ -353,7 +353,7 @@ class DeviceParams:
     """A [P][GTS_NPARAM] int32 parameter table resident on the GPU."""
 
     def __init__(self, dgraph: DeviceGraph, params, stream=None, tensor=None, n_points=None, ordered=True):
-        """``ordered``: hand points to the warps largest estimated cost first
+        """``ordered``: hand points to the warps by estimated cost, dearest first
         (gts_params_set_order); results are the same either way."""
         import torch
         self.dgraph = dgraph
