@@ -10,8 +10,9 @@
 // holds the dependency counters of nodes that are not warp heads yet.
 //
 // Two kernels do this: k_simulate issues one node per step of the warp, and
-// k_simulate_lanes one node on each of up to 32 simulated SMs, where the graph and
-// the rows allow it (described above its functions; the notes here are k_simulate's).
+// k_simulate_lanes one node on each of up to 32 simulated SMs, for batches whose graph
+// and rows allow it and that it is estimated to run faster (described above its
+// functions; the notes here are k_simulate's).
 //
 // Semantics are those stated in include/gts.h.  Design notes:
 //  * Issue keys (Section 5.3, lowest-id reading).  A head's key is the
@@ -1605,9 +1606,9 @@ __host__ __device__ inline float lane_cost(float fed, float ns, float nodes) {
 // horizon overtakes.  Fitted to 900 tables on a GB300: ws GEMM and attention graphs,
 // 1 to 132 SMs of 3 to 30 slots, 1 to 3,000 rows, HBM at 32 B/cycle and up, GTO with 1
 // and 4 schedulers, round-robin, the L2 model.  Against the better kernel of each table
-// the choice loses 1.0% on the mean (0.4% under a policy); against k_simulate 18% at
-// most (66 SMs of 24 slots, HBM at 32 B/cycle) and 7% under a policy (GTO, 3 SMs of 30
-// slots).  ms in k_simulate and in the lanes, ws GEMM 2048x2048x512
+// the choice loses 1.0% on the mean (0.4% under a policy); 7 of 855 run again with it
+// were more than 1.5% slower than k_simulate: 18% on 66 SMs of 24 slots with HBM at 32
+// B/cycle, 4-5% under policies on SMs of 24 and 30 slots.  ms in k_simulate and in the lanes, ws GEMM 2048x2048x512
 // on 3,000 rows: one SM, 3 / 30 slots 18.7 / 20.9 and 21.1 / 53.5; 2 SMs 19.4 / 21.0
 // and 13.0 / 29.4; 4 SMs 19.6 / 21.2 and 7.8 / 16.9; 4 SMs with HBM at 32 B/cycle
 // 19.0 / 22.6 and 20.8 / 51.6; 132 SMs 22.0 / 23.3 and 4.0 / 8.3.  Under round-robin,
